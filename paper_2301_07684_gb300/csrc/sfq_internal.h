@@ -48,7 +48,7 @@ struct RateLaunch {
     double pref;
     sfq_counters *counters;
     cudaStream_t stream;
-    int grid;
+    int grid, block;
     double pair_chi_min;
     int cheb = 0;            // `table` holds Chebyshev pieces (Clenshaw evaluator)
 };
@@ -59,7 +59,7 @@ struct SampleLaunch {
     const sfq_ctx *ctx;      // tables (full or truncated) of the context
     sfq_counters *counters;
     cudaStream_t stream;
-    int grid;
+    int grid, block;
 };
 struct StepLaunch {
     const sfq_ctx *ctx;
@@ -81,9 +81,9 @@ cudaError_t launch_rate_f64(const RateLaunch &, bool pair);
 cudaError_t launch_sample_f32(const SampleLaunch &, bool pair);
 cudaError_t launch_sample_f64(const SampleLaunch &, bool pair);
 cudaError_t launch_uniforms_f32(int64_t n, const uint64_t *id, uint32_t step, uint32_t tag, uint64_t seed,
-                                void *u, cudaStream_t s, int grid);
+                                void *u, cudaStream_t s, int grid, int block);
 cudaError_t launch_uniforms_f64(int64_t n, const uint64_t *id, uint32_t step, uint32_t tag, uint64_t seed,
-                                void *u, cudaStream_t s, int grid);
+                                void *u, cudaStream_t s, int grid, int block);
 cudaError_t launch_step_f32(const StepLaunch &);
 cudaError_t launch_step_f64(const StepLaunch &);
 cudaError_t launch_fused_f32(const StepLaunch &, uint32_t nsteps);

@@ -31,7 +31,7 @@ static cudaError_t launch_rate_t(const RateLaunch &L, bool pair) {
     const T *tab = static_cast<const T *>(L.table);
     auto kern = pair ? (L.cheb ? rate_kernel<T, true, true> : rate_kernel<T, true, false>)
                      : (L.cheb ? rate_kernel<T, false, true> : rate_kernel<T, false, false>);
-    kern<<<L.grid, 256, 0, L.stream>>>(L.n, g, x, out, tab, (T)L.pref, L.counters, (T)L.pair_chi_min);
+    kern<<<L.grid, L.block, 0, L.stream>>>(L.n, g, x, out, tab, (T)L.pref, L.counters, (T)L.pair_chi_min);
     return cudaGetLastError();
 }
 
@@ -46,28 +46,28 @@ static cudaError_t launch_sample_t(const SampleLaunch &L, bool pair) {
         tab.nlc_inv = static_cast<const T *>(L.ctx->d_nlc_inv_ch);
         tab.nbw_inv = static_cast<const T *>(L.ctx->d_nbw_inv_ch);
         if (pair)
-            sample_kernel<T, true, false, true><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+            sample_kernel<T, true, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
         else
-            sample_kernel<T, false, false, true><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+            sample_kernel<T, false, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
         return cudaGetLastError();
     }
     const bool tr = tab.tr > 0;
     if (pair && tr)
-        sample_kernel<T, true, true><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+        sample_kernel<T, true, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     else if (pair)
-        sample_kernel<T, true, false><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+        sample_kernel<T, true, false><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     else if (tr)
-        sample_kernel<T, false, true><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+        sample_kernel<T, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     else
-        sample_kernel<T, false, false><<<L.grid, 256, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+        sample_kernel<T, false, false><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     return cudaGetLastError();
 }
 
 template <typename T>
 static cudaError_t launch_uniforms_t(int64_t n, const uint64_t *id, uint32_t step, uint32_t tag, uint64_t seed,
-                                     void *u, cudaStream_t s, int grid) {
+                                     void *u, cudaStream_t s, int grid, int block) {
     if (n == 0) return cudaSuccess;
-    uniforms_kernel<T><<<grid, 256, 0, s>>>(n, id, step, tag, seed, static_cast<T *>(u));
+    uniforms_kernel<T><<<grid, block, 0, s>>>(n, id, step, tag, seed, static_cast<T *>(u));
     return cudaGetLastError();
 }
 

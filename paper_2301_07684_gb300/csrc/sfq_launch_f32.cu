@@ -5,8 +5,8 @@ namespace sfq {
 cudaError_t launch_rate_f32(const RateLaunch &L, bool pair) { return launch_rate_t<float>(L, pair); }
 cudaError_t launch_sample_f32(const SampleLaunch &L, bool pair) { return launch_sample_t<float>(L, pair); }
 cudaError_t launch_uniforms_f32(int64_t n, const uint64_t *id, uint32_t step, uint32_t tag, uint64_t seed, void *u,
-                                cudaStream_t s, int grid) {
-    return launch_uniforms_t<float>(n, id, step, tag, seed, u, s, grid);
+                                cudaStream_t s, int grid, int block) {
+    return launch_uniforms_t<float>(n, id, step, tag, seed, u, s, grid, block);
 }
 cudaError_t launch_step_f32(const StepLaunch &L) {
     return L.ctx->inv_tr > 0 ? launch_step_trunc_f32(L) : launch_step_t<float, false>(L);

@@ -1,0 +1,50 @@
+"""Launch rules of the entry points: the sizes at which a kernel or its launch shape changes.
+An element's result does not depend on how many elements a call has, so every size is
+compared bit for bit with one large call over the same elements."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2301_07684_gb300 import sfq
+from paper_2301_07684_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _elements(n, dtype, seed=5):
+    g = np.random.default_rng(seed)
+    dev = lambda a: torch.as_tensor(a).to(device="cuda", dtype=dtype)
+    # the whole range of both samplers and its outside, with the special values at the front
+    chi = 10.0 ** g.uniform(-5, 4, n)
+    gam = 10.0 ** g.uniform(0, 5, n)
+    r = (g.integers(0, 1 << 23, n) + 0.5) / (1 << 23)
+    chi[:6] = [0.0, np.nan, -1.0, np.inf, 4096.0, 1e-30]
+    r[6:10] = [0.0, 1.0, np.nan, 2.0 ** -24]
+    return dev(gam), dev(chi), dev(r)
+
+
+def _all(ctx, gam, chi, r, ids, counters):
+    return [ctx.uniforms(ids, 3, 1), ctx.photon_rate(gam, chi, counters=counters),
+            ctx.pair_rate(gam, chi, counters=counters), *ctx.sample_photon_xi(chi, r, counters=counters),
+            *ctx.sample_pair_xi(chi, r, counters=counters)]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_element_calls_of_every_size_agree(precision):
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision=precision, seed=4)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    big = sms * 256 * 9 + 77
+    gam, chi, r = _elements(big, ctx.dtype)
+    ids = torch.arange(big, device="cuda", dtype=torch.int64)
+    whole = _all(ctx, gam, chi, r, ids, None)
+    for n in (1, 31, 32, 33, sms * 32 - 1, sms * 32 + 1, 4096, sms * 255 + 1, sms * 256, sms * 256 * 8 + 1):
+        part = _all(ctx, gam[:n], chi[:n], r[:n], ids[:n], None)
+        for a, b in zip(part, whole):
+            assert torch.equal(a.view(torch.uint8), b[:n].contiguous().view(torch.uint8)), n
+    # the counters count every element once, whatever the shape
+    cnt = [sfq.counters_tensor() for _ in range(2)]
+    _all(ctx, gam, chi, r, ids, cnt[0])
+    for k in range(0, big, 40000):
+        s = slice(k, min(k + 40000, big))
+        _all(ctx, gam[s].clone(), chi[s].clone(), r[s].clone(), ids[s].clone(), cnt[1])
+    assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
