@@ -48,3 +48,30 @@ def test_element_calls_of_every_size_agree(precision):
         s = slice(k, min(k + 40000, big))
         _all(ctx, gam[s].clone(), chi[s].clone(), r[s].clone(), ids[s].clone(), cnt[1])
     assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
+
+
+@pytest.mark.parametrize("n", [1, 63, 65, 127 * 64, 128 * 64, 128 * 64 + 1, 257 * 64 - 3])
+def test_loss_and_gradient_around_the_reduction_chunks(n):
+    """Gradient partials are per 64 samples and reduced 128 at a time; against automatic
+    differentiation in binary64.  A gradient is a binary32 sum of at most n terms, each a
+    chain of 64-term binary32 sums: 2 (64 + 64) 2^-24 = 1.5e-5 relative to the norm covers
+    both when the errors add up."""
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision="fp32", seed=4)
+    net = sfq.Surrogate(ctx, seed=3)
+    g = np.random.default_rng(n)
+    chi = torch.as_tensor(np.exp(g.uniform(np.log(1e-3), np.log(100.0), n)).astype(np.float32)).cuda()
+    u = torch.as_tensor(((g.integers(0, 1 << 23, n) + 0.5) / (1 << 23)).astype(np.float32)).cuda()
+    lnw = net.plain_targets(chi, u)
+    loss, grad = net.loss_grad(chi, u, lnw)
+    th = torch.as_tensor(net.get_params()).cuda().double().requires_grad_()
+    c, s = 0.5 * (np.log(1e-3) + np.log(100.0)), 0.5 * (np.log(100.0) - np.log(1e-3))
+    h = torch.stack([(chi.double().log() - c) / s, -torch.log1p(-u.double()) / 8 - 1], 1)
+    at = 0
+    for k, (o, i) in enumerate([(64, 2), (64, 64), (64, 64), (1, 64)]):
+        h = h @ th[at:at + o * i].view(o, i).t() + th[at + o * i:at + o * i + o]
+        h = torch.nn.functional.silu(h) if k < 3 else h
+        at += o * i + o
+    ref = (h[:, 0] - lnw.double() + u.double().log()).square().mean()
+    ref.backward()
+    assert abs(float(loss) / float(ref.detach()) - 1) < 1.5e-5
+    assert float((grad.double() - th.grad).norm() / th.grad.norm()) < 1.5e-5
