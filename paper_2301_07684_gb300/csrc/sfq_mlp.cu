@@ -16,85 +16,10 @@
 // tolerance in u (a bound on its contribution to the KS distance of the sampled energies)
 // are flagged by sfq_mlp_calibrate; draws in flagged cells, and chi outside the training
 // range [1e-3, 100], use the plain sampler.
-#include <cmath>
-#include <cstring>
-#include <string>
-#include <vector>
-
-#include <cuda_bf16.h>
-
-#include "sfq_internal.h"
-#include "sfq_kernels.cuh"
-
-struct sfq_mlp {
-    sfq_ctx *ctx;
-    int kind;                         // 0: photon emission (Eq. again), 1: pair creation (Eq. again_pp)
-    float *params, *m, *v;            // binary32 master parameters, Adam moments
-    uint8_t *flags;                   // fallback cells (NCELL bytes)
-    float *cell_err;                  // per-cell calibration error (NCELL floats)
-    int64_t adam_t;
-    int calibrated;
-};
+#include "sfq_mlp.cuh"
 
 namespace sfq {
 namespace mlp {
-
-constexpr int H = 64;
-constexpr int NP = 8577;
-constexpr int NPS = 8592;          // row stride of the gradient partials (16-byte aligned rows)
-constexpr int O_W1 = 0, O_B1 = 128, O_W2 = 192, O_B2 = 4288, O_W3 = 4352, O_B3 = 8448, O_W4 = 8512, O_B4 = 8576;
-constexpr float C_CHI = -1.1512925464970229f;    // (ln 1e-3 + ln 100) / 2
-constexpr float S_CHI = 5.7564627324851140f;     // (ln 100 - ln 1e-3) / 2
-constexpr float L_SCALE = 0.125f;
-constexpr float CHI_LO = 1e-3f, CHI_HI = 100.0f;
-constexpr int NCX = 64, NCU = 64, NCELL = NCX * NCU;   // calibration cells in (ln chi, u)
-
-__device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-__device__ __forceinline__ float qz(float x, bool q) { return q ? bf16r(x) : x; }
-__device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
-// SiLU of the inference paths (tensor-core kernel, SIMT reference and calibration) with one
-// special-function instruction: z sigma(z) = h (1 + tanh h), h = z / 2, from
-// sigma(z) = (1 + tanh(z/2)) / 2.  tanh.approx.f32 has a relative error below 2^-10.987
-// (PTX ISA), which is below the bfloat16 rounding the activations then get (2^-9).
-// `h` is passed in: the callers form it as 0.5 z + 0.5 b in one fma from halved biases.
-__device__ __forceinline__ float silu_h(float h) {
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(h));
-    return fmaf(h, t, h);
-}
-__device__ __forceinline__ float dsilu(float z) {
-    const float s = __fdividef(1.0f, 1.0f + __expf(-z));
-    return s * (1.0f + z * (1.0f - s));
-}
-// What distinguishes the two samplers the network can stand for.  Photon emission: input
-// u = r, chi in [1e-3, 100], sampler variable ln w-bar.  Pair creation: input u = |r'| =
-// |2r - 1|, chi in [0.1, 100], sampler variable ln(-ln y) with y = 1 - v-bar (Eq.
-// again_pp): -ln y ~ v-bar ~ u as u -> 0, so both variables minus ln u stay smooth at
-// u -> 0, and y = exp(-u e^network) never exceeds 1.  The network output is always the
-// sampler variable minus ln u.
-struct Kind {
-    float c_chi, inv_s_chi, chi_lo, chi_hi;
-    int pair;
-};
-constexpr float P_C_CHI = 1.1512925464970229f;      // (ln 0.1 + ln 100) / 2
-constexpr float P_S_CHI = 3.4538776394910684f;      // (ln 100 - ln 0.1) / 2
-constexpr float P_CHI_LO = 0.1f, P_CHI_HI = 100.0f;
-inline Kind kind_of(int pair) {
-    return pair ? Kind{P_C_CHI, 1.0f / P_S_CHI, P_CHI_LO, P_CHI_HI, 1} : Kind{C_CHI, 1.0f / S_CHI, CHI_LO, CHI_HI, 0};
-}
-__device__ __forceinline__ void features(const Kind &K, float chi, float u, float &x1, float &x2) {
-    x1 = (logf(chi) - K.c_chi) * K.inv_s_chi;
-    x2 = -log1pf(-u) * L_SCALE - 1.0f;
-}
-// network output + offset = the sampler's variable (ln w-bar or ln(-ln y))
-__device__ __forceinline__ float out_offset(const Kind &, float u) { return logf(u); }
-__device__ __forceinline__ int cell_of(const Kind &K, float chi, float u) {
-    const float t = (logf(chi) - logf(K.chi_lo)) * (float)NCX / (logf(K.chi_hi) - logf(K.chi_lo));
-    int cx = (int)t, cu = (int)(u * (float)NCU);
-    cx = cx < 0 ? 0 : (cx >= NCX ? NCX - 1 : cx);
-    cu = cu < 0 ? 0 : (cu >= NCU ? NCU - 1 : cu);
-    return cx * NCU + cu;
-}
 
 // ---------------------------------------------------------------------------------------
 // Initialisation: U(-1/sqrt(fan_in), 1/sqrt(fan_in)) for weights and biases (Philox).
@@ -422,124 +347,6 @@ __global__ void __launch_bounds__(RB) reduce_kernel(const float *__restrict__ pa
     var[p] = vi;
     const float mh = mi / (1.0f - b1t), vh = vi / (1.0f - b2t);
     params[p] -= lr * mh / (sqrtf(vh) + 1e-8f);
-}
-
-// ---------------------------------------------------------------------------------------
-// SIMT forward of one sample with the weights in shared memory (calibration and the
-// reference inference path).  Same rounding as the tensor-core kernel.
-struct SimtW {
-    float w1[H * 2], b1[H], w2[H * H], b2[H], w3[H * H], b3[H], w4[H], b4;
-};
-__device__ __forceinline__ void stage_simt(SimtW &W, const float *P) {
-    for (int e = threadIdx.x; e < H * H; e += blockDim.x) {
-        W.w2[e] = bf16r(P[O_W2 + e]);
-        W.w3[e] = bf16r(P[O_W3 + e]);
-    }
-    for (int e = threadIdx.x; e < H; e += blockDim.x) {
-        W.w1[2 * e] = bf16r(P[O_W1 + 2 * e]);
-        W.w1[2 * e + 1] = bf16r(P[O_W1 + 2 * e + 1]);
-        W.b1[e] = P[O_B1 + e];
-        W.b2[e] = P[O_B2 + e];
-        W.b3[e] = P[O_B3 + e];
-        W.w4[e] = bf16r(P[O_W4 + e]);
-    }
-    if (threadIdx.x == 0) W.b4 = P[O_B4];
-}
-__device__ __forceinline__ float forward_simt(const SimtW &W, const Kind &K, float chi, float u) {
-    float x1, x2;
-    features(K, chi, u, x1, x2);
-    float a[H], b[H];
-#pragma unroll
-    for (int j = 0; j < H; ++j)
-        a[j] = bf16r(silu_h(0.5f * fmaf(W.w1[2 * j], x1, fmaf(W.w1[2 * j + 1], x2, W.b1[j]))));
-    // layers 2 and 3: the products summed in binary32 (the tensor cores' order differs), then
-    // h = (sum + b) / 2 as the tensor-core epilogue forms it
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int k = 0; k < H; ++k) acc = fmaf(a[k], W.w2[j * H + k], acc);
-        b[j] = bf16r(silu_h(fmaf(0.5f, acc, 0.5f * W.b2[j])));
-    }
-#pragma unroll
-    for (int j = 0; j < H; ++j) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int k = 0; k < H; ++k) acc = fmaf(b[k], W.w3[j * H + k], acc);
-        a[j] = bf16r(silu_h(fmaf(0.5f, acc, 0.5f * W.b3[j])));
-    }
-    float y = W.b4;
-#pragma unroll
-    for (int k = 0; k < H; ++k) y = fmaf(a[k], W.w4[k], y);
-    return y;
-}
-
-__global__ void __launch_bounds__(128) predict_kernel(const float *__restrict__ P, const Kind K, int64_t n,
-                                                      const float *__restrict__ chi, const float *__restrict__ u,
-                                                      float *__restrict__ lnw) {
-    __shared__ SimtW W;
-    stage_simt(W, P);
-    __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float uu = u[i];
-        lnw[i] = forward_simt(W, K, chi[i], uu) + out_offset(K, uu);
-    }
-}
-
-// ---------------------------------------------------------------------------------------
-// Calibration: per cell, the largest |u_net - u| implied by the network's ln w-bar against
-// the plain sampler's, |d ln w| / (d ln w / du), over 8 x 8 points of the cell.
-// The plain fitted sampler's variable: ln w-bar (photon) or ln(-ln y) (pair, u = |r'|).
-__device__ __forceinline__ float plain_lnw(const Kind &K, const float *inv, float chi, float u) {
-    bool oor = false;
-    if (K.pair) {
-        // -ln y from v-bar = 1 - y where y is near 1; where 1 - y falls below the binary32
-        // table's resolution (|r'| below about 1e-5) the variable is unresolved: NaN
-        const float y = pair_y<float>(inv, chi, u, oor);
-        const float v = 1.0f - y;
-        if (!(v >= 1.52587890625e-05f)) return __int_as_float(0x7fffffff);    // 2^-16
-        return logf(y < 0.5f ? -logf(y) : -log1pf(-v));
-    }
-    const float s = photon_s<float>(inv, chi, u, oor);
-    return (logf(2.0f * s) - logf(3.0f * chi)) * (1.0f / 3.0f);
-}
-__global__ void __launch_bounds__(64) calibrate_kernel(const float *__restrict__ P, const Kind K,
-                                                       const float *__restrict__ inv, float tol_u,
-                                                       uint8_t *__restrict__ flags, float *__restrict__ cell_err) {
-    __shared__ SimtW W;
-    __shared__ float red[64];
-    stage_simt(W, P);
-    __syncthreads();
-    const int cell = blockIdx.x, cx = cell / NCU, cu = cell % NCU;
-    const int pa = threadIdx.x >> 3, pb = threadIdx.x & 7;
-    const float lo = logf(K.chi_lo), span = logf(K.chi_hi) - logf(K.chi_lo);
-    const float chi = expf(lo + span * ((float)cx + ((float)pa + 0.5f) * 0.125f) / (float)NCX);
-    const float u = ((float)cu + ((float)pb + 0.5f) * 0.125f) / (float)NCU;
-    const float ln_net = forward_simt(W, K, chi, u) + out_offset(K, u);
-    const float ln_p = plain_lnw(K, inv, chi, u);
-    const float h = 1.0f / (float)(NCU * 64);
-    // |d ln w / du| (both sampler variables rise with u)
-    const float dlnw_du = fabsf(plain_lnw(K, inv, chi, u + h) - plain_lnw(K, inv, chi, u - h)) / (2.0f * h);
-    float e = fabsf(ln_net - ln_p) / fmaxf(dlnw_du, 1e-30f);
-    if (!(e == e)) e = 1e30f;
-    red[threadIdx.x] = e;
-    __syncthreads();
-    for (int o = 32; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + o]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        cell_err[cell] = red[0];
-        flags[cell] = red[0] > tol_u ? 1 : 0;
-    }
-}
-
-// ln w-bar of the plain fitted sampler (training targets without the oracle).
-__global__ void plain_targets_kernel(const float *__restrict__ inv, const Kind K, int64_t n,
-                                     const float *__restrict__ chi, const float *__restrict__ u,
-                                     float *__restrict__ lnw) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        lnw[i] = plain_lnw(K, inv, chi[i], u[i]);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1191,8 +998,7 @@ sfq_status sfq_mlp_predict_lnw(sfq_mlp *m, int64_t n, const float *chi, const fl
     DeviceGuard g(m->ctx->device);
     const int64_t blocks = (n + 127) / 128;
     const int grid = (int)(blocks < (int64_t)m->ctx->num_sms * 8 ? blocks : (int64_t)m->ctx->num_sms * 8);
-    predict_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>(m->params, kind_of(m->kind), n, chi, u, lnw);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_predict(m->params, kind_of(m->kind), n, chi, u, lnw, grid, (cudaStream_t)stream);
     return e == cudaSuccess ? SFQ_OK : cuda_fail(m->ctx, e, "sfq_mlp_predict_lnw");
 }
 
@@ -1204,8 +1010,8 @@ sfq_status sfq_mlp_plain_targets(sfq_mlp *m, int64_t n, const float *chi, const 
     DeviceGuard g(m->ctx->device);
     const int64_t blocks = (n + 255) / 256;
     const int grid = (int)(blocks < (int64_t)m->ctx->num_sms * 8 ? blocks : (int64_t)m->ctx->num_sms * 8);
-    plain_targets_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(inv_table(m), kind_of(m->kind), n, chi, u, lnw);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        launch_plain_targets(inv_table(m), kind_of(m->kind), n, chi, u, lnw, grid, (cudaStream_t)stream);
     return e == cudaSuccess ? SFQ_OK : cuda_fail(m->ctx, e, "sfq_mlp_plain_targets");
 }
 
@@ -1214,8 +1020,7 @@ sfq_status sfq_mlp_calibrate(sfq_mlp *m, float tol_u, int32_t *n_flagged, float 
     if (!(tol_u > 0.0f)) return fail(m->ctx, SFQ_ERR_ARG, "tol_u must be positive");
     DeviceGuard g(m->ctx->device);
     const cudaStream_t s = (cudaStream_t)stream;
-    calibrate_kernel<<<NCELL, 64, 0, s>>>(m->params, kind_of(m->kind), inv_table(m), tol_u, m->flags, m->cell_err);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_calibrate(m->params, kind_of(m->kind), inv_table(m), tol_u, m->flags, m->cell_err, s);
     std::vector<uint8_t> f(NCELL);
     std::vector<float> ce(NCELL);
     if (e == cudaSuccess) e = cudaMemcpyAsync(f.data(), m->flags, NCELL, cudaMemcpyDeviceToHost, s);
