@@ -169,6 +169,30 @@ __device__ __forceinline__ T wtilde_pair(const T *c, T chi, bool &oor, T chi_min
     return chi * h * exp_m83(chi);
 }
 
+// Pieces of the two inverse-CDF tables, and the piece of (chi, r) with its local variables.
+template <typename T>
+struct InvPieces {
+    using Q = L<T>;
+    static constexpr int PI_NX = (Q::PI_XLOW ? 1 << Q::PI_XSUBLOW : 0) + (Q::PI_XEHI - Q::PI_XELO) * (1 << Q::PI_XSUB);
+    static constexpr int PP_NX = (Q::PP_XLOW ? 1 << Q::PP_XSUBLOW : 0) + (Q::PP_XEHI - Q::PP_XELO) * (1 << Q::PP_XSUB);
+    static constexpr int PI_N = PI_NX * Q::PI_NY, PP_N = PP_NX * Q::PP_NY;
+};
+template <typename T>
+__device__ __forceinline__ int photon_piece(T chi, T r, T &xc, T &xr, bool &low, bool &oor) {
+    using Q = L<T>;
+    const int ic = octave_piece<T, Q::PI_XELO, Q::PI_XEHI, Q::PI_XSUB, Q::PI_XLOW, Q::PI_XSUBLOW>(chi, xc, oor);
+    const int ir = prob_piece<T, Q::PI_YE0, Q::PI_YSUB, Q::PI_YSUBLOW, Q::PI_YQLO, Q::PI_YSUBQ>(r, xr, low, oor);
+    return ic * Q::PI_NY + ir;
+}
+template <typename T>
+__device__ __forceinline__ int pair_piece(T chi, T a, T &xc, T &xr, bool &oor) {
+    using Q = L<T>;
+    bool low;
+    const int ic = octave_piece<T, Q::PP_XELO, Q::PP_XEHI, Q::PP_XSUB, Q::PP_XLOW, Q::PP_XSUBLOW>(chi, xc, oor);
+    const int ir = prob_piece<T, Q::PP_YE0, Q::PP_YSUB, Q::PP_YSUBLOW, Q::PP_YQLO, Q::PP_YSUBQ>(a, xr, low, oor);
+    return ic * Q::PP_NY + ir;
+}
+
 // s = 3 chi w^3 / 2 for w-bar = G~_pe(r, chi) (Eq. again, Eq. subs_altri).  TR > 0 reads the
 // table truncated by TR degrees in each variable.
 template <typename T, int TR = 0, bool CH = false>
@@ -177,9 +201,7 @@ __device__ __forceinline__ T photon_s(const T *__restrict__ inv, T chi, T r, boo
     constexpr int DX = Q::PI_DX - TR, DY = Q::PI_DY - TR;
     T xc, xr;
     bool low;
-    const int ic = octave_piece<T, Q::PI_XELO, Q::PI_XEHI, Q::PI_XSUB, Q::PI_XLOW, Q::PI_XSUBLOW>(chi, xc, oor);
-    const int ir = prob_piece<T, Q::PI_YE0, Q::PI_YSUB, Q::PI_YSUBLOW, Q::PI_YQLO, Q::PI_YSUBQ>(r, xr, low, oor);
-    const T *c = inv + ((size_t)ic * Q::PI_NY + ir) * ((DX + 1) * padded_row(DY + 1, sizeof(T)));
+    const T *c = inv + (size_t)photon_piece<T>(chi, r, xc, xr, low, oor) * ((DX + 1) * padded_row(DY + 1, sizeof(T)));
     T w = CH ? clenshaw2<DX, DY>(c, xc, xr) : horner2<DX, DY>(c, xc, xr);
     if (low) w *= r;                          // the low-r block holds w-bar / r
     const T chi_eff = chi > (T)4096 ? (T)4096 : chi;
@@ -194,10 +216,7 @@ __device__ __forceinline__ T pair_y(const T *__restrict__ inv, T chi, T a, bool 
     using Q = L<T>;
     constexpr int DX = Q::PP_DX - TR, DY = Q::PP_DY - TR;
     T xc, xr;
-    bool low;
-    const int ic = octave_piece<T, Q::PP_XELO, Q::PP_XEHI, Q::PP_XSUB, Q::PP_XLOW, Q::PP_XSUBLOW>(chi, xc, oor);
-    const int ir = prob_piece<T, Q::PP_YE0, Q::PP_YSUB, Q::PP_YSUBLOW, Q::PP_YQLO, Q::PP_YSUBQ>(a, xr, low, oor);
-    const T *c = inv + ((size_t)ic * Q::PP_NY + ir) * ((DX + 1) * padded_row(DY + 1, sizeof(T)));
+    const T *c = inv + (size_t)pair_piece<T>(chi, a, xc, xr, oor) * ((DX + 1) * padded_row(DY + 1, sizeof(T)));
     return CH ? clenshaw2<DX, DY>(c, xc, xr) : horner2<DX, DY>(c, xc, xr);
 }
 
@@ -356,6 +375,25 @@ __global__ void __launch_bounds__(256) rate_kernel(int64_t n, const T *__restric
 
 // Batched samplers (App. A functions 9 and 11, Eqs. again, again_pp).
 // CH: tab.nlc_inv / tab.nbw_inv hold Chebyshev pieces, evaluated by Clenshaw's recurrence.
+// One valid element (chi >= 0, 0 < r < 1): xi and 1 - xi, or the two leptons' shares.
+template <typename T, bool PAIR, bool TRUNC, bool CH>
+__device__ __forceinline__ void sample_one(const Tables<T> &tab, T x, T u, T &a, T &b, bool &oor) {
+    if (PAIR) {
+        if (CH) pair_shares<T, 0, true>(tab.nbw_inv, x, u, a, b, oor);
+        else pair_shares_sel<T, TRUNC>(tab, x, u, a, b, oor);
+    } else {
+        const T s = CH ? photon_s<T, 0, true>(tab.nlc_inv, x, u, oor) : photon_s_sel<T, TRUNC>(tab, x, u, oor);
+        const T inv1s = (T)1 / ((T)1 + s);
+        a = s * inv1s;                     // xi = s/(1+s)
+        b = inv1s;                         // 1 - xi
+    }
+}
+template <typename T>
+__device__ __forceinline__ bool sample_valid(T x, T u) {
+    return x >= (T)0 && u > (T)0 && u < (T)1;
+}
+
+// One element per thread: small calls, and binary64, which the FP64 pipe bounds.
 template <typename T, bool PAIR, bool TRUNC, bool CH = false>
 __global__ void __launch_bounds__(256) sample_kernel(int64_t n, const T *__restrict__ chi,
                                                      const T *__restrict__ r, T *__restrict__ out_a,
@@ -365,26 +403,207 @@ __global__ void __launch_bounds__(256) sample_kernel(int64_t n, const T *__restr
     c.zero();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const T x = chi[i], u = r[i];
-        bool oor = false;
-        if (!(x >= (T)0) || !(u > (T)0) || !(u < (T)1)) {
-            ++c.v[C_NAN];
-            out_a[i] = (T)0;
-            if (out_b) out_b[i] = (T)0;
-            continue;
-        }
-        if (PAIR) {
-            T xe, xp;
-            if (CH) pair_shares<T, 0, true>(tab.nbw_inv, x, u, xe, xp, oor);
-            else pair_shares_sel<T, TRUNC>(tab, x, u, xe, xp, oor);
-            out_a[i] = xe;
-            if (out_b) out_b[i] = xp;
+        T a = (T)0, b = (T)0;
+        if (sample_valid(x, u)) {
+            bool oor = false;
+            sample_one<T, PAIR, TRUNC, CH>(tab, x, u, a, b, oor);
+            c.v[C_OOR] += oor;
         } else {
-            const T s = CH ? photon_s<T, 0, true>(tab.nlc_inv, x, u, oor) : photon_s_sel<T, TRUNC>(tab, x, u, oor);
-            const T inv1s = (T)1 / ((T)1 + s);
-            out_a[i] = s * inv1s;          // xi = s/(1+s)
-            if (out_b) out_b[i] = inv1s;   // 1 - xi
+            ++c.v[C_NAN];
         }
-        c.v[C_OOR] += oor;
+        out_a[i] = a;
+        if (out_b) out_b[i] = b;
+    }
+    flush_counters(c, counters);
+}
+
+// Large binary32 calls.  A draw reads the 81 coefficients of its own piece of the table (27
+// loads of 16 bytes), and with random chi and r the lanes of a warp hold as many pieces as
+// lanes: sample_kernel keeps the L1 data stage 85 % busy and DRAM 6 % (478 us for 2^24
+// draws).  So each block first sorts a tile of SAMP_TILE elements by piece (a histogram in
+// shared memory, every piece's run padded to whole groups of four), and a thread evaluates
+// four draws of one piece with one load of its coefficients: 219 us (photon) and 195 us
+// (pair, from 448).  What remains is issue (59 % of the slots: 81 multiply-adds and 200 other
+// instructions per draw) and the phases' barriers.  One draw per thread from the sorted tile
+// took 280 us; blocks of 256 threads (tiles of 2048 or 4096) or 1024 took 237 to 253 us.
+constexpr int SAMP_BS = 512, SAMP_PER = 8, SAMP_TILE = SAMP_BS * SAMP_PER, SAMP_BINS = 1024;
+constexpr int SAMP_MINB = 2;                               // resident blocks per SM
+constexpr int SAMP_G = 4;                                  // draws of one piece that a thread evaluates together
+constexpr int SAMP_PIECES = InvPieces<float>::PI_N > InvPieces<float>::PP_N ? InvPieces<float>::PI_N : InvPieces<float>::PP_N;
+constexpr int SAMP_SLOTS = (SAMP_TILE + (SAMP_G - 1) * SAMP_PIECES + 7) / 8 * 8;   // the padded runs of one tile
+constexpr size_t SAMP_SMEM =
+    (size_t)SAMP_SLOTS * (2 * sizeof(float) + sizeof(uint16_t)) + (size_t)SAMP_TILE * 2 * sizeof(float) + SAMP_BINS * sizeof(uint32_t);
+static_assert(SAMP_PIECES <= SAMP_BINS && SAMP_BINS % SAMP_BS == 0, "a bin per piece; whole bins per thread");
+static_assert(SAMP_TILE < 65535, "16-bit positions; 65535 marks the padding");
+
+// Four draws of the piece of the first: the arithmetic of photon_s / pair_shares for each.
+template <bool PAIR, int TR>
+__device__ __forceinline__ void sample_group(const Tables<float> &tab, const float (&x)[SAMP_G],
+                                             const float (&u)[SAMP_G], float (&oa)[SAMP_G], float (&ob)[SAMP_G],
+                                             bool (&oor)[SAMP_G]) {
+    using Q = L<float>;
+    constexpr int DX = (PAIR ? Q::PP_DX : Q::PI_DX) - TR, DY = (PAIR ? Q::PP_DY : Q::PI_DY) - TR;
+    constexpr int ROW = padded_row(DY + 1, (int)sizeof(float));
+    float xc[SAMP_G], xr[SAMP_G], w[SAMP_G];
+    int piece = 0;
+    bool low = false;                                      // the same for a whole piece
+#pragma unroll
+    for (int j = 0; j < SAMP_G; ++j) {
+        bool lw = false;
+        const int pj = PAIR ? pair_piece<float>(x[j], fabsf(2.0f * u[j] - 1.0f), xc[j], xr[j], oor[j])
+                            : photon_piece<float>(x[j], u[j], xc[j], xr[j], lw, oor[j]);
+        if (j == 0) { piece = pj; low = lw; }
+    }
+    const float *__restrict__ c = (PAIR ? (TR ? tab.nbw_inv_r : tab.nbw_inv) : (TR ? tab.nlc_inv_r : tab.nlc_inv)) +
+                                  (size_t)piece * ((DX + 1) * ROW);
+#pragma unroll
+    for (int i = DX; i >= 0; --i) {
+        float co[ROW];
+#pragma unroll
+        for (int k = 0; k < ROW / 4; ++k) ldg_vec(c + i * ROW + 4 * k, co + 4 * k);
+#pragma unroll
+        for (int j = 0; j < SAMP_G; ++j) {
+            float b = co[DY];
+#pragma unroll
+            for (int k = DY - 1; k >= 0; --k) b = fmaf(b, xr[j], co[k]);
+            w[j] = i == DX ? b : fmaf(w[j], xc[j], b);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < SAMP_G; ++j) {
+        if (PAIR) {
+            const float small = 0.5f * w[j], big = 1.0f - small;
+            const bool pos = 2.0f * u[j] - 1.0f >= 0.0f;
+            oa[j] = pos ? big : small;
+            ob[j] = pos ? small : big;
+        } else {
+            const float wj = low ? w[j] * u[j] : w[j];
+            const float chi_eff = x[j] > 4096.0f ? 4096.0f : x[j];
+            const float s = 1.5f * chi_eff * wj * wj * wj;
+            const float inv1s = 1.0f / (1.0f + s);
+            oa[j] = s * inv1s;
+            ob[j] = inv1s;
+        }
+    }
+}
+
+template <bool PAIR, int TR>
+__global__ void __launch_bounds__(SAMP_BS, SAMP_MINB)
+    sample_tile_kernel(int64_t n, const float *__restrict__ chi, const float *__restrict__ r,
+                       float *__restrict__ out_a, float *__restrict__ out_b, const Tables<float> tab,
+                       sfq_counters *counters) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    float *s_chi = reinterpret_cast<float *>(smem), *s_r = s_chi + SAMP_SLOTS, *s_a = s_r + SAMP_SLOTS,
+          *s_b = s_a + SAMP_TILE;
+    uint32_t *bin = reinterpret_cast<uint32_t *>(s_b + SAMP_TILE);
+    uint16_t *s_at = reinterpret_cast<uint16_t *>(bin + SAMP_BINS);
+    __shared__ uint32_t wsum[SAMP_BS / 32];
+    constexpr int BPT = SAMP_BINS / SAMP_BS;               // bins per thread of the scan
+    constexpr uint32_t NONE = 0xFFFFFFFFu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    Cnt c;
+    c.zero();
+    for (int k = 0; k < BPT; ++k) bin[k * SAMP_BS + tid] = 0u;
+    const int64_t ntiles = (n + SAMP_TILE - 1) / SAMP_TILE;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int64_t base = t * SAMP_TILE;
+        float x[SAMP_PER], u[SAMP_PER];
+        uint32_t key[SAMP_PER];                            // rank within the piece << 10 | piece
+        __syncthreads();                                   // the bins are zero, the last tile is stored
+#pragma unroll
+        for (int k = 0; k < SAMP_PER; ++k) {
+            const int64_t i = base + k * SAMP_BS + tid;
+            x[k] = u[k] = -1.0f;
+            if (i < n) { x[k] = chi[i]; u[k] = r[i]; }
+        }
+#pragma unroll
+        for (int k = 0; k < SAMP_PER; ++k) {
+            key[k] = NONE;
+            if (sample_valid(x[k], u[k])) {
+                float xc, xr;
+                bool low, oor;
+                const int p = PAIR ? pair_piece<float>(x[k], fabsf(2.0f * u[k] - 1.0f), xc, xr, oor)
+                                   : photon_piece<float>(x[k], u[k], xc, xr, low, oor);
+                key[k] = atomicAdd(&bin[p], 1u) << 10 | (uint32_t)p;
+            } else if (base + k * SAMP_BS + tid < n) {
+                ++c.v[C_NAN];                              // NaN or invalid: zeros
+                s_a[k * SAMP_BS + tid] = 0.0f;
+                s_b[k * SAMP_BS + tid] = 0.0f;
+            }
+        }
+        __syncthreads();
+        // exclusive scan of the padded runs (BPT consecutive bins per thread)
+        uint32_t cnt[BPT], sum = 0;
+#pragma unroll
+        for (int k = 0; k < BPT; ++k) {
+            cnt[k] = bin[tid * BPT + k];
+            sum += (cnt[k] + SAMP_G - 1) / SAMP_G * SAMP_G;
+        }
+        uint32_t inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        uint32_t off = inc - sum, total = 0;
+#pragma unroll
+        for (int w = 0; w < SAMP_BS / 32; ++w) {
+            const uint32_t v = wsum[w];
+            off += w < warp ? v : 0u;
+            total += v;
+        }
+#pragma unroll
+        for (int k = 0; k < BPT; ++k) {
+            bin[tid * BPT + k] = off;
+            const uint32_t end = off + (cnt[k] + SAMP_G - 1) / SAMP_G * SAMP_G;
+            for (uint32_t e = off + cnt[k]; e < end; ++e) {       // at most SAMP_G - 1 slots of padding
+                s_chi[e] = 1.0f;
+                s_r[e] = 0.5f;
+                s_at[e] = 0xFFFFu;
+            }
+            off = end;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < SAMP_PER; ++k) {
+            if (key[k] != NONE) {
+                const uint32_t at = bin[key[k] & (SAMP_BINS - 1)] + (key[k] >> 10);
+                s_chi[at] = x[k];
+                s_r[at] = u[k];
+                s_at[at] = (uint16_t)(k * SAMP_BS + tid);
+            }
+        }
+        __syncthreads();
+        for (int k = 0; k < BPT; ++k) bin[k * SAMP_BS + tid] = 0u;
+        for (uint32_t g = tid; g < total / SAMP_G; g += SAMP_BS) {
+            const float4 xv = *reinterpret_cast<const float4 *>(s_chi + SAMP_G * g);
+            const float4 uv = *reinterpret_cast<const float4 *>(s_r + SAMP_G * g);
+            const ushort4 av = *reinterpret_cast<const ushort4 *>(s_at + SAMP_G * g);
+            const float xg[SAMP_G] = {xv.x, xv.y, xv.z, xv.w}, ug[SAMP_G] = {uv.x, uv.y, uv.z, uv.w};
+            const uint32_t to[SAMP_G] = {av.x, av.y, av.z, av.w};
+            float a[SAMP_G], b[SAMP_G];
+            bool oor[SAMP_G] = {};
+            sample_group<PAIR, TR>(tab, xg, ug, a, b, oor);
+#pragma unroll
+            for (int j = 0; j < SAMP_G; ++j) {
+                if (to[j] != 0xFFFFu) {
+                    s_a[to[j]] = a[j];
+                    s_b[to[j]] = b[j];
+                    c.v[C_OOR] += oor[j];
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < SAMP_PER; ++k) {
+            const int64_t i = base + k * SAMP_BS + tid;
+            if (i < n) {
+                out_a[i] = s_a[k * SAMP_BS + tid];
+                if (out_b) out_b[i] = s_b[k * SAMP_BS + tid];
+            }
+        }
     }
     flush_counters(c, counters);
 }

@@ -35,32 +35,51 @@ static cudaError_t launch_rate_t(const RateLaunch &L, bool pair) {
     return cudaGetLastError();
 }
 
-template <typename T>
-static cudaError_t launch_sample_t(const SampleLaunch &L, bool pair) {
-    if (L.n == 0) return cudaSuccess;
+template <bool PAIR, int TR>
+static cudaError_t launch_sample_tile(const SampleLaunch &L, const Tables<float> &tab) {
+    auto kern = sample_tile_kernel<PAIR, TR>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SAMP_SMEM);
+    if (e != cudaSuccess) return e;
+    const int64_t ntiles = (L.n + SAMP_TILE - 1) / SAMP_TILE, wave = (int64_t)SAMP_MINB * L.ctx->num_sms;
+    kern<<<(unsigned)(ntiles < wave ? ntiles : wave), SAMP_BS, SAMP_SMEM, L.stream>>>(
+        L.n, static_cast<const float *>(L.chi), static_cast<const float *>(L.r), static_cast<float *>(L.a),
+        static_cast<float *>(L.b), tab, L.counters);
+    return cudaGetLastError();
+}
+
+template <typename T, bool PAIR>
+static cudaError_t launch_sample_k(const SampleLaunch &L, Tables<T> tab) {
     const T *x = static_cast<const T *>(L.chi), *r = static_cast<const T *>(L.r);
     T *a = static_cast<T *>(L.a), *b = static_cast<T *>(L.b);
-    Tables<T> tab = tables_of<T>(L.ctx);
-    if (L.ctx->eval == SFQ_EVAL_CLENSHAW) {
+    const bool clenshaw = L.ctx->eval == SFQ_EVAL_CLENSHAW;
+    if constexpr (sizeof(T) == 4) {
+        // sorted tiles once every SM has one (at that size 25 us one element per thread, under
+        // 16 us sorted); smaller calls, which tiles would leave SMs idle in, and the comparison
+        // evaluator take one element per thread
+        if (!clenshaw && L.n >= (int64_t)SAMP_TILE * L.ctx->num_sms) {
+            if (tab.tr == 2) return launch_sample_tile<PAIR, 2>(L, tab);
+            if (tab.tr == 1) return launch_sample_tile<PAIR, 1>(L, tab);
+            return launch_sample_tile<PAIR, 0>(L, tab);
+        }
+    }
+    if (clenshaw) {
         // the comparison evaluator: Chebyshev pieces of the full tables, Clenshaw's recurrence
         tab.nlc_inv = static_cast<const T *>(L.ctx->d_nlc_inv_ch);
         tab.nbw_inv = static_cast<const T *>(L.ctx->d_nbw_inv_ch);
-        if (pair)
-            sample_kernel<T, true, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
-        else
-            sample_kernel<T, false, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
-        return cudaGetLastError();
+        sample_kernel<T, PAIR, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+    } else if (tab.tr > 0) {
+        sample_kernel<T, PAIR, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
+    } else {
+        sample_kernel<T, PAIR, false><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     }
-    const bool tr = tab.tr > 0;
-    if (pair && tr)
-        sample_kernel<T, true, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
-    else if (pair)
-        sample_kernel<T, true, false><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
-    else if (tr)
-        sample_kernel<T, false, true><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
-    else
-        sample_kernel<T, false, false><<<L.grid, L.block, 0, L.stream>>>(L.n, x, r, a, b, tab, L.counters);
     return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t launch_sample_t(const SampleLaunch &L, bool pair) {
+    if (L.n == 0) return cudaSuccess;
+    const Tables<T> tab = tables_of<T>(L.ctx);
+    return pair ? launch_sample_k<T, true>(L, tab) : launch_sample_k<T, false>(L, tab);
 }
 
 template <typename T>

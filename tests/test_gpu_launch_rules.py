@@ -50,6 +50,33 @@ def test_element_calls_of_every_size_agree(precision):
     assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
 
 
+@pytest.mark.parametrize("k", [9, 8, 7])
+def test_sorted_sampler_tiles(k):
+    """Binary32 sampler calls sort tiles of 4096 elements once every SM has a tile: the draws
+    and counters of calls around that size equal those of calls below it, with the full and
+    the truncated tables, with every element in one piece and with an unused second output."""
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision="fp32", seed=4)
+    ctx.set_sampler_coefficients(k)
+    line = torch.cuda.get_device_properties(0).multi_processor_count * 4096
+    big = 2 * line + 1
+    _, chi, r = _elements(big, ctx.dtype, seed=k)
+    one = torch.full_like(chi, 1.3), torch.full_like(r, 0.3)
+    for x, u in ((chi, r), one):
+        cnt = [sfq.counters_tensor() for _ in range(2)]
+        parts = [(ctx.sample_photon_xi(x[a:a + 99328], u[a:a + 99328], counters=cnt[0]),
+                  ctx.sample_pair_xi(x[a:a + 99328], u[a:a + 99328], counters=cnt[0])) for a in range(0, big, 99328)]
+        small = [torch.cat([p[i][j] for p in parts]) for i in (0, 1) for j in (0, 1)]
+        for n in (line - 1, line, line + 1, line + 4095, big):
+            c = cnt[1] if n == big else None
+            whole = [*ctx.sample_photon_xi(x[:n], u[:n], counters=c), *ctx.sample_pair_xi(x[:n], u[:n], counters=c)]
+            for a, b in zip(whole, small):
+                assert torch.equal(a.view(torch.int32), b[:n].view(torch.int32)), n
+        assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
+    xi = torch.empty_like(chi)
+    st = sfq.lib().sfq_sample_photon_xi(ctx._h, big, sfq._ptr(chi), sfq._ptr(r), sfq._ptr(xi), None, None, sfq._stream())
+    assert st == 0 and torch.equal(xi, ctx.sample_photon_xi(chi, r)[0])
+
+
 @pytest.mark.parametrize("n", [1, 63, 65, 127 * 64, 128 * 64, 128 * 64 + 1, 257 * 64 - 3])
 def test_loss_and_gradient_around_the_reduction_chunks(n):
     """Gradient partials are per 64 samples and reduced 128 at a time; against automatic
