@@ -77,6 +77,61 @@ def test_sorted_sampler_tiles(k):
     assert st == 0 and torch.equal(xi, ctx.sample_photon_xi(chi, r)[0])
 
 
+def _sort_keys(kind, n, g):
+    """(parent id, step, meta) of one form of records; the step and meta bits that differ and
+    the parent-id bits that differ decide the sort's path."""
+    meta = np.full(n, 2, np.uint8)                              # a photon of a primary
+    step = g.integers(0, 200, n).astype(np.uint32)
+    pid = g.integers(0, max(n // 3, 1), n).astype(np.uint64)
+    if kind == "pairs":
+        member = g.integers(0, 3, n)
+        meta = (np.array([2, 0, 1])[member] | member << 2 | g.integers(0, 3, n) << 4 | g.integers(0, 4, n) << 6).astype(np.uint8)
+    elif kind == "same":
+        step[:], pid[:] = 7, 1 << 40
+    elif kind == "offset":                                      # a rank's id range, late steps
+        step, pid = step + np.uint32(0xFFFFFF00), pid + np.uint64((1 << 50) + 12345)
+    elif kind == "hashed":                                      # a cascade's descendants: 64 bits
+        pid = g.integers(0, 1 << 63, n, dtype=np.uint64) * np.uint64(2) + np.uint64(1)
+        step = g.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+    elif kind.startswith("width"):                              # exactly so many differing bits
+        w = int(kind[5:]) - 6                                   # steps 0 .. 3, members and tags: 6 bits
+        pid = g.integers(0, 1 << w, n, dtype=np.uint64)
+        pid[:2] = 0, (1 << w) - 1
+        step = g.integers(0, 4, n).astype(np.uint32)
+        meta = (g.integers(0, 64, n)).astype(np.uint8)
+        step[:2], meta[:2] = (0, 3), (0, 63)
+    return pid, step, meta
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("kind", ["photons", "pairs", "same", "offset", "hashed", "width32", "width33", "width64",
+                                  "width65"])
+def test_sort_paths(kind, precision):
+    """The one-block sort, the composite keys of 32 and 64 bits and the two stages, at the edges
+    of a block's records, of tiles and of the one-block path, against numpy's stable sort of
+    every column; the scratch-free call alike."""
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision=precision, seed=4)
+    g = np.random.default_rng(len(kind))
+    for n in (2, 33, 1023, 1025, 16383, 16384, 16385, 5 * 4096, 5 * 4096 + 1, 300001):
+        pid, step, meta = _sort_keys(kind, n, g)
+        p = g.standard_normal((3, n))
+        order = np.lexsort(((meta >> 4) & 3, (meta >> 2) & 3, step, pid))
+        for noalloc in (False, True):
+            out = sfq.ProductBuffers(n + 5, ctx.dtype, "cuda")
+            for t, a in zip((out.px, out.py, out.pz, out.parent_id, out.step, out.meta),
+                            (*p, pid.view(np.int64), step.view(np.int32), meta)):
+                t[:n] = torch.as_tensor(a).to(device="cuda", dtype=t.dtype)
+                t[n:] = 77
+            out.count[0] = n
+            (ctx.sort_products_noalloc if noalloc else ctx.sort_products)(out)
+            r = out.to_numpy()
+            assert all((t[n:] == 77).all() for t in (out.px, out.parent_id, out.step, out.meta))
+            assert np.array_equal(r["parent_id"], pid[order]) and np.array_equal(r["step"], step[order]), (n, noalloc)
+            assert np.array_equal(r["meta"], meta[order]), (n, noalloc)
+            for k, a in zip(("px", "py", "pz"), p):
+                assert np.array_equal(r[k], a.astype(r[k].dtype)[order]), (n, noalloc)
+
+
 @pytest.mark.parametrize("n", [1, 63, 65, 127 * 64, 128 * 64, 128 * 64 + 1, 257 * 64 - 3])
 def test_loss_and_gradient_around_the_reduction_chunks(n):
     """Gradient partials are per 64 samples and reduced 128 at a time; against automatic
