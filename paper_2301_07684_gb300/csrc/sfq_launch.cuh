@@ -95,6 +95,13 @@ static cudaError_t launch_uniforms_t(int64_t n, const uint64_t *id, uint32_t ste
 // The TMA-staged shapes compiled with the truncated samplers (TRUNC) are limited to 16
 // consumer warps; the warp-streaming ones to 2 particles per lane.
 constexpr int TRUNC_CW = 16, TRUNC_PPT = 2;
+// Consumer warps per block of the default shape.  With the producer they are 20 or 16 warps, 5
+// or 4 per scheduler, which leaves 96 or 128 registers a thread (16 consumer warps: 17, five
+// on one scheduler).  Fields in memory wait on HBM and on event batches, where more warps
+// help: 8 steps of 2^24 particles 1539 us with 19, 1552 with 15, 1574 with 23 (80 registers).
+// The plane wave is bound by issue: 40 steps of 4.2e6 particles 2058 us with 15, 2085 with 19,
+// 2191 with 23.
+constexpr int TMA_CW_SOA = 19, TMA_CW_PW = 15;
 
 template <typename T, bool TRUNC>
 static cudaError_t prepare_step_t() {
@@ -114,6 +121,12 @@ static cudaError_t prepare_step_t() {
         SFQ_PREP(8)
         SFQ_PREP(16)
         SFQ_PREP(20)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>());
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_PW, TMA_CW_PW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)tma_smem_bytes<T, FK_PW, TMA_CW_PW>());
     }
 #undef SFQ_PREP
     if (e == cudaSuccess) done = true;
@@ -202,8 +215,8 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
     const bool pw = f.kind == SFQ_FIELDS_PLANE_WAVE;
     // TMA-staged kernel: one persistent block per SM; chosen automatically when every
     // SM gets at least one full tile.  `ppt` selects the consumer warps per block.
-    const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : 16);
-    const int tile = cw * (sizeof(T) == 4 ? 64 : 32);
+    const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : (pw ? TMA_CW_PW : TMA_CW_SOA));
+    const int tile = (cw < 16 ? cw : 16) * (sizeof(T) == 4 ? 64 : 32);
     // the beyond-LCFA model runs on the warp-streaming kernel (its state is read directly)
     const bool tma = !L.cascade && p.lepton_model == SFQ_LEPTON_LCFA_OD &&
                      (L.variant == 2 || (L.variant == 0 && p.n >= (int64_t)tile * ctx->num_sms));
@@ -223,9 +236,16 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
         } else {
             switch (cw) {
                 SFQ_TMA_CASE(8)
-                SFQ_TMA_CASE(20)
-                default:
                 SFQ_TMA_CASE(16)
+                SFQ_TMA_CASE(20)
+                case TMA_CW_PW:
+                    kern = mc_step_tma_kernel<T, FK_PW, TMA_CW_PW>;
+                    smem = tma_smem_bytes<T, FK_PW, TMA_CW_PW>();
+                    break;
+                default:
+                    kern = mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>;
+                    smem = tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>();
+                    break;
             }
         }
 #undef SFQ_TMA_CASE

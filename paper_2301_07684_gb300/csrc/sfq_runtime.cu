@@ -219,8 +219,8 @@ sfq_status sfq_autotune_step(sfq_ctx *ctx, const sfq_particles *p, const sfq_fie
         return st;
     }
     struct Shape { int variant, ppt; };
-    const Shape shapes[6] = {{1, 1}, {1, 2}, {1, 4}, {2, 8}, {2, 16}, {2, 20}};
-    const int nshapes = blcfa ? 3 : 6;           // the beyond-LCFA model runs on the warp-streaming kernel
+    const Shape shapes[7] = {{1, 1}, {1, 2}, {1, 4}, {2, 8}, {2, 16}, {2, 20}, {2, 0}};
+    const int nshapes = blcfa ? 3 : 7;           // the beyond-LCFA model runs on the warp-streaming kernel
     const int saved[3] = {ctx->step_variant, ctx->step_ppt, ctx->step_grid};
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     e = cudaEventCreate(&ev0);

@@ -71,7 +71,7 @@ struct StepArgs {
 // Entry of the TMA-staged kernel's event queue: the particle's state as the step read it,
 // so that the event path re-reads nothing from global memory.
 template <typename T>
-struct QEntry {
+struct __align__(16) QEntry {
     int64_t i;          // particle index
     T g;                // energy of the particle
     T chi;              // quantum parameter at the event
@@ -340,6 +340,20 @@ __device__ __forceinline__ void reserve_records(unsigned long long *ocount, unsi
     bs = __shfl_sync(0xFFFFFFFFu, b1, 31) + (unsigned long long)(pre_s - nspawn);
 }
 
+// The same for a batch in which no lane writes more than one record or creates more than one
+// child (no converted photon): two ballots instead of a prefix sum.
+__device__ __forceinline__ void reserve_single(unsigned long long *ocount, unsigned long long *scount, bool prod,
+                                               bool spawn, unsigned long long &bp, unsigned long long &bs) {
+    const int lane = threadIdx.x & 31;
+    const unsigned mp = __ballot_sync(0xFFFFFFFFu, prod), ms = __ballot_sync(0xFFFFFFFFu, spawn);
+    unsigned long long v = 0;
+    if (lane == 0 && mp) v = atomicAdd(ocount, (unsigned long long)__popc(mp));
+    if (lane == 1 && ms) v = atomicAdd(scount, (unsigned long long)__popc(ms));
+    const unsigned lt = (1u << lane) - 1u;
+    bp = __shfl_sync(0xFFFFFFFFu, v, 0) + (unsigned long long)__popc(mp & lt);
+    bs = ms ? __shfl_sync(0xFFFFFFFFu, v, 1) + (unsigned long long)__popc(ms & lt) : 0ull;
+}
+
 // One batch of up to 32 queued events, one per lane (lanes with valid = false idle); all
 // 32 lanes execute it (warp shuffles).  The lane receives the particle's index i, its
 // energy g, chi at the event, aux (-1 for an optical-depth event; for beyond-LCFA,
@@ -348,7 +362,9 @@ __device__ __forceinline__ void reserve_records(unsigned long long *ocount, unsi
 // global atomic per batch, before the sampling when every record count is known up
 // front (no beyond-LCFA lane, whose emission may be rejected), so that the atomic's
 // latency overlaps the sampling.
-template <typename T, bool TRUNC = false, bool CASC = false, bool SURR = false>
+// SINGLE: batches without a converted photon take the ballot reservation (the TMA-staged
+// kernel; the warp-streaming instances, held to 64 registers, lost 3 % to the extra code).
+template <typename T, bool TRUNC = false, bool CASC = false, bool SURR = false, bool SINGLE = false>
 __device__ __forceinline__ void process_events_core(const StepArgs<T> &a, uint32_t step, int64_t ei, T eg, T echi,
                                                     T e_aux, T px, T py, T pz, uint8_t fl, bool valid, Cnt &c,
                                                     EvOut<T> &o) {
@@ -371,7 +387,10 @@ __device__ __forceinline__ void process_events_core(const StepArgs<T> &a, uint32
     // spawned particles: the pair of a converted photon; in a cascade also the emitted photon
     int nspawn = a.scount ? (photon ? 2 : (CASC ? nprod : 0)) : 0;
     unsigned long long bp = 0, bs = 0;
-    if (!late) reserve_records(a.ocount, a.scount, nprod, nspawn, bp, bs);
+    if (!late) {
+        if (!SINGLE || __any_sync(0xFFFFFFFFu, photon)) reserve_records(a.ocount, a.scount, nprod, nspawn, bp, bs);
+        else reserve_single(a.ocount, a.scount, nprod != 0, nspawn != 0, bp, bs);
+    }
     T xa = 0, xb = 0;
     uint64_t id = 0;
     uint32_t tag = 0;
@@ -519,11 +538,11 @@ __device__ __forceinline__ void process_events_core(const StepArgs<T> &a, uint32
 
 // process_events_core at the launch's step with the parent's new state stored to the
 // population in global memory.
-template <typename T, bool TRUNC = false, bool CASC = false, bool SURR = false>
+template <typename T, bool TRUNC = false, bool CASC = false, bool SURR = false, bool SINGLE = false>
 __device__ __forceinline__ void process_events(const StepArgs<T> &a, int64_t ei, T eg, T echi, T e_aux, T px,
                                                T py, T pz, uint8_t fl, bool valid, Cnt &c) {
     EvOut<T> o;
-    process_events_core<T, TRUNC, CASC, SURR>(a, a.step, ei, eg, echi, e_aux, px, py, pz, fl, valid, c, o);
+    process_events_core<T, TRUNC, CASC, SURR, SINGLE>(a, a.step, ei, eg, echi, e_aux, px, py, pz, fl, valid, c, o);
     if (o.what & 1) { a.px[ei] = o.px; a.py[ei] = o.py; a.pz[ei] = o.pz; }
     if (o.what & 2) a.tau[ei] = o.tau;
     if (o.what & 4) a.flags[ei] = o.fl;
@@ -591,41 +610,115 @@ __device__ __forceinline__ bool step_particle_v(const StepArgs<T> &a, const T *s
     return od_update(&tau, d, a.seed, id_of, step, (fl >> SFQ_TAG_SHIFT) & 3u);
 }
 
-// Two alive leptons of one lane, binary32: the arithmetic of step_particle_v for each,
-// written as one block with the rare optical-depth draw in front, so that nothing
-// branches between the two dependency chains and they interleave.  The NaN guard of
-// step_particle_v becomes a select (the rate is evaluated at chi = 0 and discarded).
-template <bool PW>
-__device__ __forceinline__ void step_lepton_pair(const StepArgs<float> &a, const float *s_nlc, int64_t i0,
-                                                 const uint8_t fl[2], const float px[2], const float py[2],
-                                                 const float pz[2], const float E[2][3], const float B[2][3],
-                                                 double tau[2], float g[2], float chi[2], bool ev[2], Cnt &c) {
-    uint64_t b[2];
+// W~_rad(chi) as wtilde_rad, without branches: the first piece and the octaves are told apart by
+// selects (binary32 tables: one piece below 2^ELO, one per octave).  high: chi beyond the table.
+__device__ __forceinline__ float wtilde_rad_sel(const float *c, float chi, bool &high) {
+    using Q = L<float>;
+    static_assert(Q::NLC_LOW == 1 && Q::NLC_SUBLOW == 0 && Q::NLC_SUB == 0, "one low piece, one piece per octave");
+    constexpr int LAST = Q::NLC_EHI - Q::NLC_ELO, ST = RateSmem<float>::NLC_STRIDE;
+    const uint32_t b = __float_as_uint(chi);
+    const int e = (int)(b >> 23) - (127 + Q::NLC_ELO - 1);        // piece of an octave: 1 ... LAST
+    high = e > LAST;
+    const int p = max(0, min(e, LAST));
+    const float m = __uint_as_float((b & 0x7FFFFFu) | 0x3F800000u);
+    const float x_oct = fmaf(2.0f, m, -3.0f), x_low = fmaf(chi, 2.0f * pow2<float>(-Q::NLC_ELO), -1.0f);
+    const float x = high ? 1.0f : (e < 1 ? x_low : x_oct);
+    return horner_smem<Q::NLC_DEG, ST>(c + p * ST, x);
+}
+
+// W~_pair(chi) as wtilde_pair, without branches (binary32: one piece per octave, none below).
+__device__ __forceinline__ float wtilde_pair_sel(const float *c, float chi, bool &out, float chi_min) {
+    using Q = L<float>;
+    static_assert(Q::NBW_LOW == 0 && Q::NBW_SUB == 0, "one piece per octave");
+    constexpr int LAST = Q::NBW_EHI - Q::NBW_ELO - 1, ST = RateSmem<float>::NBW_STRIDE;
+    const bool on = chi >= chi_min;
+    const float v = on ? chi : chi_min;
+    const uint32_t b = __float_as_uint(v);
+    const int e = (int)(b >> 23) - (127 + Q::NBW_ELO);
+    out = on && (e < 0 || e > LAST);
+    const float x_oct = fmaf(2.0f, __uint_as_float((b & 0x7FFFFFu) | 0x3F800000u), -3.0f);
+    const float x = e > LAST ? 1.0f : (e < 0 ? -1.0f : x_oct);
+    const float w = v * horner_smem<Q::NBW_DEG, ST>(c + max(0, min(e, LAST)) * ST, x) * exp_m83(v);
+    return on ? w : 0.0f;
+}
+
+// Two alive leptons of one lane, or (PHOTON) two particles that are each a photon or dead,
+// binary32: the arithmetic of step_particle_v for the alive ones, operation for operation, with
+// both in packed registers (f32x2) up to the rate's piece and without a branch but the rare
+// optical-depth draw in front.  Photons die as they convert: the dead ride along masked, so
+// that a population's warps stay in one path (with a block for two alive photons only, warps
+// ran it and the general path: 31 us against 27 for 1e6 photons of which a third has
+// converted).  Leptons rarely do, and the mask cost them 3 % of a plane-wave step.
+// E[1] alone is read with the plane wave; tab is the species' rate table.
+template <bool PW, bool PHOTON>
+__device__ __forceinline__ void step_pair(const StepArgs<float> &a, const float *tab, int64_t i0, uint32_t fl2,
+                                          f32x2 px, f32x2 py, f32x2 pz, const f32x2 E[3], const f32x2 B[3],
+                                          double tau[2], float g[2], float chi[2], bool ev[2], Cnt &c) {
+    const bool on[2] = {!PHOTON || (fl2 & SFQ_ALIVE) != 0u, !PHOTON || (fl2 & (SFQ_ALIVE << 8)) != 0u};
+    uint64_t b[2] = {(uint64_t)__double_as_longlong(tau[0]), (uint64_t)__double_as_longlong(tau[1])};
+    if (PHOTON ? (on[0] && (int64_t)b[0] < 0) || (on[1] && (int64_t)b[1] < 0) : (int64_t)(b[0] | b[1]) < 0) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const auto id_of = [&]() { return a.id ? a.id[i0 + k] : a.id_base + (uint64_t)(i0 + k); };
-        b[k] = od_fill((uint64_t)__double_as_longlong(tau[k]), a.seed, id_of, a.step, (fl[k] >> SFQ_TAG_SHIFT) & 3u);
+        for (int k = 0; k < 2; ++k) {
+            const auto id_of = [&]() { return a.id ? a.id[i0 + k] : a.id_base + (uint64_t)(i0 + k); };
+            if (on[k]) b[k] = od_fill(b[k], a.seed, id_of, a.step, (fl2 >> (8 * k + SFQ_TAG_SHIFT)) & 3u);
+        }
     }
+    const f32x2 one(1.0f, 1.0f), half(0.5f, 0.5f);
+    const f32x2 p2 = fma2(px, px, fma2(py, py, mul2(pz, pz)));
+    const f32x2 g2 = PHOTON ? p2 : add2(one, p2);                  // leptons: >= 1, or NaN
+    float q0, q1;
+    g2.get(q0, q1);
+    const f32x2 r = PHOTON ? f32x2(rsqrtf(q0), rsqrtf(q1)) : f32x2(rsqrt_normal(q0), rsqrt_normal(q1));
+    f32x2 inv_g = fma2(mul2(half, r), fma2(mul2(g2, r), neg2(r), one), r);            // rsqrt_nr
+    if (PHOTON) {
+        float r0, r1;
+        inv_g.get(r0, r1);
+        inv_g = f32x2(q0 > 0.0f ? r0 : 0.0f, q1 > 0.0f ? r1 : 0.0f);
+    }
+    const f32x2 gg = mul2(g2, inv_g);
+    f32x2 q;
+    if (PW) {
+        const f32x2 fx = mul2(py, E[1]), fy = fma2(gg, E[1], mul2(neg2(px), E[1]));  // chi_pw
+        q = fma2(mul2(fx, fx), f32x2(-1.0f, -1.0f), fma2(fx, fx, mul2(fy, fy)));
+    } else {
+        const f32x2 nx = neg2(px), ny = neg2(py), nz = neg2(pz);                      // chi_of
+        const f32x2 fx = fma2(gg, E[0], fma2(py, B[2], mul2(nz, B[1])));
+        const f32x2 fy = fma2(gg, E[1], fma2(pz, B[0], mul2(nx, B[2])));
+        const f32x2 fz = fma2(gg, E[2], fma2(px, B[1], mul2(ny, B[0])));
+        const f32x2 pe = fma2(px, E[0], fma2(py, E[1], mul2(pz, E[2])));
+        q = fma2(neg2(pe), pe, fma2(fx, fx, fma2(fy, fy, mul2(fz, fz))));
+    }
+    q.get(q0, q1);
+    const f32x2 rq(rsqrtf(q0), rsqrtf(q1)), sq = mul2(q, rq);      // sqrt_nr; 0 for q <= 0 or NaN
+    float c0, c1;
+    fma2(mul2(half, rq), fma2(neg2(sq), sq, q), sq).get(c0, c1);
+    const f32x2 cc = mul2(f32x2(q0 > 0.0f ? c0 : 0.0f, q1 > 0.0f ? c1 : 0.0f), f32x2(a.inv_rho, a.inv_rho));
+    cc.get(chi[0], chi[1]);
+    gg.get(g[0], g[1]);
+    bool out[2];
     float d[2];
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const float p2 = fmaf(px[k], px[k], fmaf(py[k], py[k], pz[k] * pz[k]));
-        const float g2 = 1.0f + p2;
-        const float inv_g = g2 > 0.0f ? rsqrt_nr(g2) : 0.0f;
-        g[k] = g2 * inv_g;
-        chi[k] = PW ? chi_pw<float>(g[k], px[k], py[k], E[k][1], a.inv_rho)
-                    : chi_of<float>(g[k], px[k], py[k], pz[k], E[k], B[k], a.inv_rho);
-        const bool ok = chi[k] >= 0.0f && g[k] > 0.0f;
-        bool oor = false;
-        const float w = wtilde_rad<float>(s_nlc, ok ? chi[k] : 0.0f, oor);
-        d[k] = ok ? a.prefdt * (chi[k] * inv_g) * w : 0.0f;
-        c.v[C_UPD] += 1;
-        c.v[C_NAN] += !ok;
-        c.v[C_OOR] += ok && oor;
-        c.v[C_RDT] += d[k] > 0.1f;
+    const f32x2 pd(a.prefdt, a.prefdt);
+    if (PHOTON) {
+        const f32x2 w(wtilde_pair_sel(tab, chi[0], out[0], a.pair_chi_min),
+                      wtilde_pair_sel(tab, chi[1], out[1], a.pair_chi_min));
+        mul2(mul2(pd, w), inv_g).get(d[0], d[1]);
+    } else {
+        const f32x2 w(wtilde_rad_sel(tab, chi[0], out[0]), wtilde_rad_sel(tab, chi[1], out[1]));
+        mul2(mul2(pd, mul2(cc, inv_g)), w).get(d[0], d[1]);
     }
 #pragma unroll
-    for (int k = 0; k < 2; ++k) ev[k] = od_sub(&tau[k], b[k], d[k]);
+    for (int k = 0; k < 2; ++k) {
+        const bool ok = chi[k] >= 0.0f && g[k] > 0.0f;
+        d[k] = ok ? d[k] : 0.0f;
+        c.v[C_UPD] += on[k];
+        c.v[C_NAN] += on[k] && !ok;
+        c.v[C_OOR] += on[k] && ok && out[k];
+        c.v[C_RDT] += on[k] && d[k] > 0.1f;
+        double t = tau[k];
+        const bool e = od_sub(&t, b[k], d[k]);
+        ev[k] = on[k] && e;
+        if (on[k]) tau[k] = t;
+    }
 }
 
 // T: float (mixed) or double; FK: field source; PPT: particles per lane per chunk.

@@ -2,12 +2,19 @@
 //
 // One persistent CTA per SM: a producer warp copies each tile's structure-of-arrays
 // slices (momenta, optical depth, flags, fields or phase index) from global to
-// shared memory with 1D bulk copies (cp.async.bulk), NSTAGE tiles ahead, and 16
+// shared memory with 1D bulk copies (cp.async.bulk), NSTAGE tiles ahead, and the
 // consumer warps compute the step (Sec. 2 and 4 of Montefiori & Tamburini,
-// arXiv:2301.07684) from shared memory.  A tile is cut into one slice per consumer warp;
+// arXiv:2301.07684) from shared memory.  A tile is cut into slices of 32 or 64 particles;
 // with fields in memory the warps claim the slices in order from a shared counter, so a
 // warp busy with its events delays no stage's release.  Each consumer warp queues its event particles, with the
-// state it read, in a ring of its own and samples them 32 at a time.  Stages are handed over with mbarriers
+// state it read, in a ring of its own and samples them 32 at a time.
+// What bounds it (binary32): with fields in memory 53 B per particle from and to HBM, about
+// 59 with the 32-byte sectors of the momenta that events rewrite; 2^24 particles take 180 us,
+// 81 % of the copy bandwidth on those bytes.  The plane wave, and populations too small to
+// fill the stages many times, are bound by issue: two leptons of a lane are stepped in
+// packed registers without branches (step_pair), 6.5 warp-instructions per particle
+// with its events (8.2 before, when 4.2e6 particles took 57 us under the profiler with fields
+// in memory and 57 with the wave; now 45 and 47).  Stages are handed over with mbarriers
 // (full: producer -> consumers, completed by the copies' transaction bytes;
 // empty: consumers -> producer).  Every wait is bounded: on a timeout the kernel
 // raises the timeout word of the counters and leaves its loops after its copies
@@ -33,6 +40,22 @@ __device__ __forceinline__ void mbar_arrive_tx(uint64_t *bar, uint32_t bytes) {
                  "r"(bytes)
                  : "memory");
 }
+// The arrival of a warp's lane 0, predicated (a branch of one lane costs the warp a
+// reconvergence).
+__device__ __forceinline__ void mbar_arrive_lane0(uint64_t *bar, int lane) {
+    asm volatile("{\n .reg .b64 st;\n .reg .pred p;\n setp.eq.s32 p, %1, 0;\n"
+                 " @p mbarrier.arrive.shared::cta.b64 st, [%0];\n}" ::"r"(smem_u32(bar)), "r"(lane)
+                 : "memory");
+}
+// The block's next slice for the warp, from a shared counter.
+__device__ __forceinline__ unsigned claim_slice(unsigned *ctr, int lane) {
+    unsigned g = 0;
+    asm volatile("{\n .reg .pred p;\n setp.eq.s32 p, %2, 0;\n @p atom.shared.add.u32 %0, [%1], 1;\n}"
+                 : "+r"(g)
+                 : "r"(smem_u32(ctr)), "r"(lane)
+                 : "memory");
+    return __shfl_sync(0xFFFFFFFFu, g, 0);
+}
 // Bounded wait for the phase of parity `parity` to complete: at most `limit` polls.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32_t limit = TMA_WAIT_LIMIT) {
     const uint32_t a = smem_u32(bar);
@@ -54,10 +77,13 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-// Layout of one stage for TILE particles.
+// Layout of one stage: a tile of SLICES slices, each one warp's work (2 particles per lane in
+// binary32, 1 in binary64).  A block of up to 16 consumer warps has a slice per warp; more
+// warps share tiles of 16 slices, so that the stages leave room for their event queues.
 template <typename T, int FK, int CW>
 struct TmaStage {
-    static constexpr int TILE = CW * (sizeof(T) == 4 ? 64 : 32);     // 2 (binary32) or 1 particle per lane
+    static constexpr int SLICES = CW < 16 ? CW : 16;
+    static constexpr int TILE = SLICES * (sizeof(T) == 4 ? 64 : 32);
     static constexpr int NF = FK == FK_SOA ? 6 : 0;
     static constexpr size_t O_PX = 0, O_PY = O_PX + TILE * sizeof(T), O_PZ = O_PY + TILE * sizeof(T);
     static constexpr size_t O_TAU = O_PZ + TILE * sizeof(T);
@@ -69,13 +95,13 @@ struct TmaStage {
 };
 
 // Dynamic shared memory of one CTA: NSTAGE stages, then the consumer warps' event queues
-// (QS entries each: one tile's events plus a partial batch), then the mbarriers.  Three
+// (QS entries each: one slice's events plus a partial batch), then the mbarriers.  Three
 // stages where they fit beside the queues and the static rate tables, else two.
 template <typename T, int FK, int CW>
 struct TmaCfg {
     using S = TmaStage<T, FK, CW>;
-    static constexpr int PPL = S::TILE / CW / 32;                  // particles per lane per tile
-    static constexpr int QS = 32 * (PPL + 1) <= 64 ? 64 : (32 * (PPL + 1) <= 128 ? 128 : 256);
+    static constexpr int PPL = S::TILE / S::SLICES / 32;           // particles per lane per slice
+    static constexpr int QS = 32 * (PPL + 1);                      // one slice's events plus a partial batch
     static constexpr size_t QBYTES = (size_t)CW * QS * sizeof(QEntry<T>);
     static constexpr size_t STATIC = (RateSmem<T>::NLC_N + RateSmem<T>::NBW_N) * sizeof(T);
     static constexpr size_t LIMIT = 227 * 1024;                    // shared memory per CTA
@@ -119,9 +145,10 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     constexpr int TMA_CONSUMER_WARPS = CW;
     constexpr int TMA_THREADS = 32 * (CW + 1);
     constexpr int TILE = S::TILE;
-    constexpr int PER_WARP = TILE / TMA_CONSUMER_WARPS;    // particles per consumer warp per tile
-    constexpr int PPL = CFG::PPL;                          // particles per lane per tile
-    constexpr int QS = CFG::QS;                            // one tile + a partial batch
+    constexpr int SLICES = S::SLICES;
+    constexpr int PER_WARP = TILE / SLICES;                // particles per slice
+    constexpr int PPL = CFG::PPL;                          // particles per lane per slice
+    constexpr int QS = CFG::QS;                            // one slice + a partial batch
     constexpr bool PAIRED = sizeof(T) == 4 && PPL == 2;     // adjacent-pair vector layout
     extern __shared__ __align__(128) unsigned char smem[];
     QEntry<T> *wq = reinterpret_cast<QEntry<T> *>(smem + CFG::O_Q);
@@ -141,7 +168,7 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     if (threadIdx.x == 0) {
         for (int s = 0; s < TMA_NSTAGE; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], TMA_CONSUMER_WARPS);
+            mbar_init(&empty[s], SLICES);
         }
         *abort_flag = 0;
         *slice_ctr = 0;
@@ -156,9 +183,8 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     if (warp == TMA_CONSUMER_WARPS) {
         // ------------------------------------------------------------- producer
         if (lane == 0) {
-            int issued_last[TMA_NSTAGE];
-            for (int s = 0; s < TMA_NSTAGE; ++s) issued_last[s] = -1;
-            for (int t = 0;; ++t) {
+            int t = 0;
+            for (;; ++t) {
                 const int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
                 if (tile >= ntiles || *(volatile int *)abort_flag) break;
                 const int s = t % TMA_NSTAGE;
@@ -190,17 +216,16 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
                 } else {
                     mbar_arrive(&full[s]);          // partial tile: consumers read global memory
                 }
-                issued_last[s] = t;
             }
             // before leaving, every copy this warp issued has landed; a drain that times out is
             // counted (the step's results are then invalid) and waited for once more, so that the
             // block does not exit while its copies may still be writing its shared memory
-            for (int s = 0; s < TMA_NSTAGE; ++s) {
-                if (issued_last[s] < 0) continue;
-                const uint32_t par = (issued_last[s] / TMA_NSTAGE) & 1;
-                if (!mbar_wait(&full[s], par)) {
+            for (int last = t > TMA_NSTAGE ? t - TMA_NSTAGE : 0; last < t; ++last) {   // the last tiles issued
+                uint64_t *bar = &full[last % TMA_NSTAGE];
+                const uint32_t par = (last / TMA_NSTAGE) & 1;
+                if (!mbar_wait(bar, par)) {
                     raise_timeout(a.counters);
-                    mbar_wait(&full[s], par);
+                    mbar_wait(bar, par);
                 }
             }
         }
@@ -209,24 +234,26 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
 
     // ------------------------------------------------------------------ consumers
     QEntry<T> *q = wq + (size_t)warp * QS;
-    unsigned head = 0, tail = 0;
+    unsigned head = 0, pend = 0;                           // ring start and entries (pend < 32 between slices)
     Cnt c;
     c.zero();
     // With fields in memory (SoA) the step waits on HBM and on its events: a warp takes the
     // block's next slice (one warp's share, PER_WARP particles, of tile t) from a shared
     // counter, so a warp that is sampling its events leaves the next slices to the others
     // instead of holding up the release of their stage.  Slices are claimed in order and each
-    // warp holds one claim, so no warp can wait on a stage two phases ahead.  With the plane
-    // wave the step is bound by issue, and warp w keeps slice w of every tile (no claim).
+    // warp holds one claim, so no warp can wait on a stage two phases ahead: the slices of
+    // the NSTAGE tiles before that phase (at least 2 x 16) would all have to be held by
+    // warps waiting for them, besides the one that keeps the stage.  With the plane wave the
+    // step is bound by issue, and the warps take the slices in turn (no claim); a warp's next
+    // slice is then at most two tiles ahead of its last, and again less than two phases.
     constexpr bool CLAIM = FK == FK_SOA;
     for (unsigned it = 0;; ++it) {
         unsigned g = it * TMA_CONSUMER_WARPS + (unsigned)warp;
         if constexpr (CLAIM) {
-            if (lane == 0) g = atomicAdd(slice_ctr, 1u);
-            g = __shfl_sync(0xFFFFFFFFu, g, 0);
+            g = claim_slice(slice_ctr, lane);
         }
-        const unsigned t = g / TMA_CONSUMER_WARPS;
-        const int sl = (int)(g % TMA_CONSUMER_WARPS);
+        const unsigned t = g / SLICES;
+        const int sl = (int)(g % SLICES);
         const int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
         if (tile >= ntiles) break;
         const int s = (int)(t % TMA_NSTAGE);
@@ -249,73 +276,65 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
         if (staged && PAIRED) {
             // full tile, binary32: lane takes the adjacent particles li0, li0 + 1 (vector loads)
             const int li0 = sl * PER_WARP + 2 * lane;
-            const float2 vx = *reinterpret_cast<const float2 *>(spx + li0);
-            const float2 vy = *reinterpret_cast<const float2 *>(spy + li0);
-            const float2 vz = *reinterpret_cast<const float2 *>(spz + li0);
+            const auto two = [&](const T *col) { return f32x2(*reinterpret_cast<const uint64_t *>(col + li0)); };
+            const f32x2 vx = two(spx), vy = two(spy), vz = two(spz);
             const double2 vt = *reinterpret_cast<const double2 *>(stau + li0);
-            const uint16_t vf = *reinterpret_cast<const uint16_t *>(sfl + li0);
-            float2 vE[3], vB[3];
-            if (FK == FK_SOA) {
-                const float *sf = reinterpret_cast<const float *>(st + S::O_F);
+            const uint32_t vf = *reinterpret_cast<const uint16_t *>(sfl + li0);
+            const T *sf = reinterpret_cast<const T *>(st + S::O_F);
+            f32x2 E2[3], B2[3];
+            if constexpr (FK == FK_SOA && PAIRED) {
 #pragma unroll
                 for (int c3 = 0; c3 < 3; ++c3) {
-                    vE[c3] = *reinterpret_cast<const float2 *>(sf + c3 * TILE + li0);
-                    vB[c3] = *reinterpret_cast<const float2 *>(sf + (3 + c3) * TILE + li0);
+                    E2[c3] = two(sf + c3 * TILE);
+                    B2[c3] = two(sf + (3 + c3) * TILE);
                 }
-            }
-            double tau_out[2] = {vt.x, vt.y};
-            // the fields of particle li0 + k
-            const auto fields = [&](int k, T E[3], T B[3]) {
-                if (FK == FK_SOA) {
+            } else if constexpr (PAIRED) {
+                T f[2];
 #pragma unroll
-                    for (int c3 = 0; c3 < 3; ++c3) {
-                        E[c3] = k == 0 ? vE[c3].x : vE[c3].y;
-                        B[c3] = k == 0 ? vB[c3].x : vB[c3].y;
-                    }
-                } else {
+                for (int k = 0; k < 2; ++k) {
                     uint32_t kk = reinterpret_cast<const uint32_t *>(st + S::O_K0)[li0 + k] + a.pw_offset;
                     kk -= (kk >= a.n_table) ? a.n_table : 0u;
                     kk = kk < a.n_table ? kk : a.n_table - 1u;
                     const T amp = has_amp ? reinterpret_cast<const T *>(st + S::O_AMP)[li0 + k] : a.amp0;
-                    const T f = amp * __ldg(a.pw_table + kk);
-                    E[0] = (T)0; E[1] = f; E[2] = (T)0;
-                    B[0] = (T)0; B[1] = (T)0; B[2] = f;
+                    f[k] = amp * __ldg(a.pw_table + kk);
                 }
-            };
-            const uint8_t fl2[2] = {(uint8_t)(vf & 0xFF), (uint8_t)(vf >> 8)};
-            const auto lepton = [](uint8_t fl) {
-                return (fl & SFQ_ALIVE) && ((fl >> SFQ_SPECIES_SHIFT) & 3) != SFQ_PHOTON;
-            };
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                pk[k][0] = k == 0 ? vx.x : vx.y;
-                pk[k][1] = k == 0 ? vy.x : vy.y;
-                pk[k][2] = k == 0 ? vz.x : vz.y;
-                fk[k] = fl2[k];
+                E2[0] = E2[2] = B2[0] = B2[1] = f32x2(0ull);
+                E2[1] = B2[2] = f32x2(f[0], f[1]);
             }
-            bool done = false;
+            double tau_out[2] = {vt.x, vt.y};
             if constexpr (PAIRED) {
-                if (lepton(fl2[0]) && lepton(fl2[1])) {
-                    // the common case: two alive leptons, stepped as one straight-line block
-                    T E2[2][3], B2[2][3];
-                    fields(0, E2[0], B2[0]);
-                    fields(1, E2[1], B2[1]);
-                    const T px2[2] = {vx.x, vx.y}, py2[2] = {vy.x, vy.y}, pz2[2] = {vz.x, vz.y};
-                    step_lepton_pair<FK == FK_PW>(a, s_nlc, start + li0, fl2, px2, py2, pz2, E2, B2, tau_out, gk,
-                                                  ck, ev, c);
-                    done = true;
-                }
+                vx.get(pk[0][0], pk[1][0]);
+                vy.get(pk[0][1], pk[1][1]);
+                vz.get(pk[0][2], pk[1][2]);
             }
-            if (!done) {
+            fk[0] = (uint8_t)(vf & 0xFFu);
+            fk[PPL - 1] = (uint8_t)(vf >> 8);
+            // two alive leptons; else no alive lepton (photons, dead); else the general path
+            constexpr uint32_t AL = SFQ_ALIVE * 0x0101u, SP = 3u << SFQ_SPECIES_SHIFT,
+                               PH = (SFQ_PHOTON << SFQ_SPECIES_SHIFT) * 0x0101u;
+            const uint32_t sx = vf ^ PH;                   // a zero species field: photon
+            const bool lep0 = (vf & SFQ_ALIVE) && (sx & SP), lep1 = (vf & (SFQ_ALIVE << 8)) && (sx & (SP << 8));
+            if ((vf & AL) == AL && (sx & SP) && (sx & (SP << 8))) {
+                if constexpr (PAIRED)
+                    step_pair<FK == FK_PW, false>(a, s_nlc, start + li0, vf, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
+            } else if (!lep0 && !lep1) {
+                if constexpr (PAIRED)
+                    step_pair<FK == FK_PW, true>(a, s_nbw, start + li0, vf, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
+            } else if constexpr (PAIRED) {
+                T e2[3][2], b2[3][2];
+#pragma unroll
+                for (int c3 = 0; c3 < 3; ++c3) {
+                    E2[c3].get(e2[c3][0], e2[c3][1]);
+                    B2[c3].get(b2[c3][0], b2[c3][1]);
+                }
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     ev[k] = false;
                     gk[k] = (T)0;
                     ck[k] = (T)0;
-                    if (fl2[k] & SFQ_ALIVE) {
-                        T E[3], B[3];
-                        fields(k, E, B);
-                        ev[k] = step_particle_v<T, FK == FK_PW>(a, s_nlc, s_nbw, start + li0 + k, fl2[k], pk[k][0],
+                    if (fk[k] & SFQ_ALIVE) {
+                        const T E[3] = {e2[0][k], e2[1][k], e2[2][k]}, B[3] = {b2[0][k], b2[1][k], b2[2][k]};
+                        ev[k] = step_particle_v<T, FK == FK_PW>(a, s_nlc, s_nbw, start + li0 + k, fk[k], pk[k][0],
                                                                 pk[k][1], pk[k][2], E, B, tau_out[k], gk[k], ck[k],
                                                                 c, a.step);
                     }
@@ -394,24 +413,27 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
                 e.py = pk[k][1];
                 e.pz = pk[k][2];
                 e.fl = fk[k];
-                q[(tail + r) & (QS - 1)] = e;
+                const unsigned at = head + pend + r;
+                q[at < (unsigned)QS ? at : at - (unsigned)QS] = e;
             }
-            tail += __popc(m);
+            pend += __popc(m);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);        // this slice of the stage is done
-        while (tail - head >= 32u) {
-            const QEntry<T> e = q[(head + lane) & (QS - 1)];
+        mbar_arrive_lane0(&empty[s], lane);           // this slice of the stage is done
+        while (pend >= 32u) {
+            const unsigned at = head + lane;
+            const QEntry<T> e = q[at < (unsigned)QS ? at : at - (unsigned)QS];
             __syncwarp();
-            head += 32;
-            process_events<T, TRUNC, false, SURR>(a, e.i, e.g, e.chi, (T)-1, e.px, e.py, e.pz, (uint8_t)e.fl, true, c);
+            head = head + 32u < (unsigned)QS ? head + 32u : 0u;   // QS is a multiple of 32, and so is head
+            pend -= 32u;
+            process_events<T, TRUNC, false, SURR, true>(a, e.i, e.g, e.chi, (T)-1, e.px, e.py, e.pz, (uint8_t)e.fl, true, c);
         }
     }
     __syncwarp();
-    if (tail != head) {
-        const unsigned nv = tail - head;
-        const QEntry<T> e = q[(head + lane) & (QS - 1)];
-        process_events<T, TRUNC, false, SURR>(a, e.i, e.g, e.chi, (T)-1, e.px, e.py, e.pz, (uint8_t)e.fl, (unsigned)lane < nv,
+    if (pend) {
+        const unsigned nv = pend, at = head + lane;
+        const QEntry<T> e = q[at < (unsigned)QS ? at : at - (unsigned)QS];
+        process_events<T, TRUNC, false, SURR, true>(a, e.i, e.g, e.chi, (T)-1, e.px, e.py, e.pz, (uint8_t)e.fl, (unsigned)lane < nv,
                                  c);
     }
     // counters of the consumer warps (the producer warp has returned)
