@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(RB) reduce_kernel(const float *__restrict__ pa
 // chunk j) at ((g * 8) + j) * 128 bytes, i.e. K-adjacent core matrices 128 bytes apart
 // (leading byte offset) and row groups 1024 bytes apart (stride byte offset).
 constexpr uint32_t MMA_WAIT_LIMIT = 1u << 22;
-constexpr int IT = 128;                       // samples per tile
-constexpr uint32_t TMEM_COLS = 64;
+constexpr int IT = 128;                       // threads of a block, rows of an activation operand
+constexpr int IS = 2 * IT;                    // samples per tile: two per thread
+constexpr uint32_t TMEM_COLS = 128;           // an accumulator of 64 columns for each
 // kind::f16 instruction descriptor: D f32 (bit 4), A bf16 (bits 7-9 = 1), B bf16 (bits
 // 10-12 = 1), both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);
@@ -404,21 +405,25 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_u32(bar))
                  : "memory");
 }
-// 32 consecutive fp32 columns of this thread's lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
-    uint32_t r[32];
+// 16 consecutive fp32 columns of this thread's lane, of two accumulators (one wait for both).
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t *r) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15}, [%16];"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr)
         : "memory");
+}
+__device__ __forceinline__ void tmem_ld16x2(uint32_t t0, uint32_t t1, float (&v)[2][16]) {
+    uint32_t r[2][16];
+    tmem_ld16(t0, r[0]);
+    tmem_ld16(t1, r[1]);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = __uint_as_float(r[k]);
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[h][k] = __uint_as_float(r[h][k]);
 }
 // Column 0 of this thread's lane.
 __device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
@@ -472,50 +477,78 @@ __device__ __forceinline__ unsigned long long warp_reserve(unsigned long long *c
     return base + (unsigned long long)__popc(m & ((1u << lane) - 1u));
 }
 
-// Operands (no-swizzle K-major, 16-byte aligned): A 128 x 64, W2 and W3 64 x 64, W4 16 x 64;
+// Operands (no-swizzle K-major, 16-byte aligned): A 128 x 64 for each half of the tile, W2 and W3 64 x 64, W4 16 x 64;
 // then layer 1's weights, the halved biases of layers 2 and 3, b4 and the fallback flags.
-constexpr uint32_t SM_A = 0, SM_B2 = 16384, SM_B3 = 24576, SM_B4 = 32768, SM_SMALL = 34816;
+constexpr uint32_t SM_A = 0, SM_A1 = 16384, SM_B2 = 32768, SM_B3 = SM_B2 + 8192, SM_B4 = SM_B3 + 8192,
+                   SM_SMALL = SM_B4 + 2048;
 constexpr uint32_t SM_FLAGS = SM_SMALL + ((H * 2 + 3 * H + 1) * 4 + 15) / 16 * 16;
 constexpr uint32_t SM_BYTES = SM_FLAGS + NCELL / 8;    // the fallback flags as one bit per cell
 constexpr uint32_t INFER_SMEM = SM_BYTES + 128;      // + alignment slack
 #ifndef SFQ_INFER_MINB
-#define SFQ_INFER_MINB 6
+#define SFQ_INFER_MINB 4
 #endif
-constexpr int INFER_MINB = SFQ_INFER_MINB;            // resident blocks per SM (registers, 36 KB of shared memory each)
+constexpr int INFER_MINB = SFQ_INFER_MINB;            // resident blocks per SM (registers, 53 KB of shared memory, 128 of 512 TMEM columns each)
 
-// Eight bfloat16 (one 16-byte K chunk of an operand row) from eight binary32 values.
-__device__ __forceinline__ uint4 pack8_bf16(const float *a) {
-    uint4 v;
-    __nv_bfloat162 p0 = __floats2bfloat162_rn(a[0], a[1]);
-    __nv_bfloat162 p1 = __floats2bfloat162_rn(a[2], a[3]);
-    __nv_bfloat162 p2 = __floats2bfloat162_rn(a[4], a[5]);
-    __nv_bfloat162 p3 = __floats2bfloat162_rn(a[6], a[7]);
-    v.x = *reinterpret_cast<uint32_t *>(&p0);
-    v.y = *reinterpret_cast<uint32_t *>(&p1);
-    v.z = *reinterpret_cast<uint32_t *>(&p2);
-    v.w = *reinterpret_cast<uint32_t *>(&p3);
-    return v;
+// SiLU of two units in packed registers: silu_h for each, one multiply-add for both.
+__device__ __forceinline__ f32x2 silu_h2(f32x2 h) {
+    float a, b, ta, tb;
+    h.get(a, b);
+    asm("tanh.approx.f32 %0, %1;" : "=f"(ta) : "f"(a));
+    asm("tanh.approx.f32 %0, %1;" : "=f"(tb) : "f"(b));
+    return fma2(h, f32x2(ta, tb), h);
+}
+// Eight bfloat16 (one 16-byte K chunk of an operand row) from four pairs.
+__device__ __forceinline__ uint32_t pack_bf16(f32x2 v) {
+    float a, b;
+    v.get(a, b);
+    __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&p);
+}
+__device__ __forceinline__ uint4 pack8_bf16(const f32x2 *v) {
+    return make_uint4(pack_bf16(v[0]), pack_bf16(v[1]), pack_bf16(v[2]), pack_bf16(v[3]));
+}
+// Four consecutive binary32 values as two pairs (a broadcast from shared memory).
+__device__ __forceinline__ void lds_pairs(const float *p, f32x2 &a, f32x2 &b) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+    a = f32x2((uint64_t)v.x);
+    b = f32x2((uint64_t)v.y);
 }
 
-// The epilogue of a hidden tensor-core layer for this thread's row, 32 accumulator columns
-// at a time (so that no more than 32 accumulators are live): h = (d + b) / 2 from the
-// halved biases hb, SiLU, and the bfloat16 row of the next layer's operand A.
+// The epilogue of a hidden tensor-core layer for this thread's two rows, 16 accumulator columns
+// of each at a time: h = (d + b) / 2 from the halved biases hb (one load for both rows),
+// SiLU, and the bfloat16 rows of the next layer's operands.
 __device__ __forceinline__ void epilogue(uint32_t t_row, const float *hb, unsigned char *a_base, int row) {
+    const f32x2 half2(0.5f, 0.5f);
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        float d[32];
-        tmem_ld32(t_row + 32 * half, d);
+    for (int part = 0; part < 4; ++part) {
+        float d[2][16];
+        tmem_ld16x2(t_row + 16 * part, t_row + 64 + 16 * part, d);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) d[j] = silu_h(fmaf(0.5f, d[j], hb[32 * half + j]));
+        for (int c = 0; c < 2; ++c) {
+            f32x2 b[4];
+            lds_pairs(hb + 16 * part + 8 * c, b[0], b[1]);
+            lds_pairs(hb + 16 * part + 8 * c + 4, b[2], b[3]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            *reinterpret_cast<uint4 *>(a_base + row_chunk_offset(row, 4 * half + c)) = pack8_bf16(d + 8 * c);
+            for (int h = 0; h < 2; ++h) {
+                f32x2 v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    v[q] = silu_h2(fma2(half2, f32x2(d[h][8 * c + 2 * q], d[h][8 * c + 2 * q + 1]), b[q]));
+                *reinterpret_cast<uint4 *>(a_base + h * (SM_A1 - SM_A) + row_chunk_offset(row, 2 * part + c)) = pack8_bf16(v);
+            }
+        }
     }
 }
 
-// One block of 128 threads walks over tiles of 128 samples (one sample per thread, one
-// row of the 128 x 64 activation tile); INFER_MINB blocks share an SM, so that the tensor
-// cores of one block's layer run while the others compute their SiLU epilogues.
+// One block of 128 threads walks over tiles of 256 samples (two per thread, a row of each of
+// two 128 x 64 activation operands); INFER_MINB blocks share an SM, so that the tensor
+// cores of one block's layer run while the others compute their SiLU epilogues.  The
+// epilogues bound it: 192 tanh per draw keep the special-function pipe 69 % busy (611 us for
+// 1e7 draws; at 100 % they would take 422).  A weight or bias that every lane reads costs the
+// shared-memory pipe as much as 32 different ones, so one read serves both samples (39 % of
+// that pipe; 58 % with one sample per thread, 618 us), and packed registers halve the
+// multiply-adds (1314 -> 943 instructions per draw and warp).  Letting the halves alternate,
+// each with its own MMA group in flight, was slower (660 us: twice the barriers).
 // APPLY (photon kind): the samples are the queued emissions of a Monte Carlo step; each
 // sampled xi also recoils its emitter (Sec. 3: the lepton keeps (1 - xi) gamma along its
 // direction) and appends the collinear photon's record.
@@ -524,7 +557,6 @@ __global__ void __launch_bounds__(IT, INFER_MINB) infer_tc_kernel(const InferArg
     extern __shared__ unsigned char sraw[];
     __shared__ uint64_t mbar;
     __shared__ uint32_t tmem_base;
-    __shared__ int s_err;
     __shared__ unsigned long long s_cnt[6];
     // 128-byte aligned operand area (the no-swizzle layout needs 16-byte alignment)
     const uint32_t raw = s_u32(sraw);
@@ -552,8 +584,8 @@ __global__ void __launch_bounds__(IT, INFER_MINB) infer_tc_kernel(const InferArg
     }
     for (int e = tid; e < H; e += IT) {
         // layer 1 halved as well (exact: a power of two), so that h = z / 2 comes out of its fmas
-        w1[2 * e] = 0.5f * bf16r(P[O_W1 + 2 * e]);
-        w1[2 * e + 1] = 0.5f * bf16r(P[O_W1 + 2 * e + 1]);
+        w1[e] = 0.5f * bf16r(P[O_W1 + 2 * e]);
+        w1[H + e] = 0.5f * bf16r(P[O_W1 + 2 * e + 1]);
         b1[e] = 0.5f * P[O_B1 + e];
         hb2[e] = 0.5f * P[O_B2 + e];
         hb3[e] = 0.5f * P[O_B3 + e];
@@ -574,7 +606,6 @@ __global__ void __launch_bounds__(IT, INFER_MINB) infer_tc_kernel(const InferArg
     }
     if (tid == 0) {
         mbar_init1(&mbar);
-        s_err = 0;
     }
     fence_async_smem();
     tc_fence_before();
@@ -589,151 +620,177 @@ __global__ void __launch_bounds__(IT, INFER_MINB) infer_tc_kernel(const InferArg
         const int64_t q = (int64_t)*a.n_dev;
         n_all = q < n_all ? q : n_all;
     }
-    const int64_t ntiles = (n_all + IT - 1) / IT;
-    int pending = 0;                              // an MMA group issued and not yet waited for
+    const int64_t ntiles = (n_all + IS - 1) / IS;
+    int late = 0;                                 // this thread gave up waiting for an MMA group
 
     // the inputs of the block's next tile are loaded a tile ahead, so that their latency falls
     // in the current tile's work
-    float chi_n = 1.0f, r_n = 0.5f;
-    {
-        const int64_t i0 = (int64_t)blockIdx.x * IT + tid;
-        if (i0 < n_all) { chi_n = a.chi[i0]; r_n = a.r[i0]; }
-    }
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t i = tile * IT + tid;
-        const bool valid = i < n_all;
-        const float chi = chi_n, r = r_n;
-        {
-            const int64_t inext = (tile + gridDim.x) * IT + tid;
-            chi_n = 1.0f;
-            r_n = 0.5f;
-            if (inext < n_all) { chi_n = a.chi[inext]; r_n = a.r[inext]; }
+    float chi_n[2], r_n[2];
+    const auto fetch = [&](int64_t tile) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t i = tile * IS + h * IT + tid;
+            chi_n[h] = 1.0f;
+            r_n[h] = 0.5f;
+            if (i < n_all) { chi_n[h] = a.chi[i]; r_n[h] = a.r[i]; }
         }
-        const bool bad = !(chi >= 0.0f) || !(r > 0.0f) || !(r < 1.0f);
-        const float rp = 2.0f * r - 1.0f;                 // pair creation: r' (exact for r in (0, 1))
-        const float u = a.K.pair ? fabsf(rp) : r;
-        const bool in_range = chi >= a.K.chi_lo && chi <= a.K.chi_hi;
-        const int cell = cell_of(a.K, chi, u);
-        const bool fallback = !bad && (!in_range || ((fl[cell >> 5] >> (cell & 31)) & 1u));
-        // layer 1 on the CUDA cores (binary32 features, bf16-rounded weights), 8 columns at a time
-        float x1, x2;
-        features(a.K, in_range ? chi : 1.0f, bad ? 0.5f : u, x1, x2);
+    };
+    fetch(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        float chi[2], r[2], u[2], x1[2], x2[2];
+        bool bad[2], fallback[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { chi[h] = chi_n[h]; r[h] = r_n[h]; }
+        fetch(tile + gridDim.x);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            bad[h] = !(chi[h] >= 0.0f) || !(r[h] > 0.0f) || !(r[h] < 1.0f);
+            u[h] = a.K.pair ? fabsf(2.0f * r[h] - 1.0f) : r[h];   // pair creation: |r'| (exact for r in (0, 1))
+            const bool in_range = chi[h] >= a.K.chi_lo && chi[h] <= a.K.chi_hi;
+            const int cell = cell_of(a.K, chi[h], u[h]);
+            fallback[h] = !bad[h] && (!in_range || ((fl[cell >> 5] >> (cell & 31)) & 1u));
+            features(a.K, in_range ? chi[h] : 1.0f, bad[h] ? 0.5f : u[h], x1[h], x2[h]);
+        }
+        // layer 1 on the CUDA cores (binary32 features, bf16-rounded weights), 8 columns at a
+        // time, the weights loaded once for both samples
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-            float v[8];
+            f32x2 wa[4], wb[4], b[4];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int j = 8 * c + q;
-                v[q] = silu_h(fmaf(w1[2 * j], x1, fmaf(w1[2 * j + 1], x2, b1[j])));
+            for (int q = 0; q < 2; ++q) {
+                lds_pairs(w1 + 8 * c + 4 * q, wa[2 * q], wa[2 * q + 1]);
+                lds_pairs(w1 + H + 8 * c + 4 * q, wb[2 * q], wb[2 * q + 1]);
+                lds_pairs(b1 + 8 * c + 4 * q, b[2 * q], b[2 * q + 1]);
             }
-            *reinterpret_cast<uint4 *>(sm + SM_A + row_chunk_offset(tid, c)) = pack8_bf16(v);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const f32x2 x11(x1[h], x1[h]), x22(x2[h], x2[h]);
+                f32x2 v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = silu_h2(fma2(wa[q], x11, fma2(wb[q], x22, b[q])));
+                *reinterpret_cast<uint4 *>(sm + SM_A + h * (SM_A1 - SM_A) + row_chunk_offset(tid, c)) = pack8_bf16(v);
+            }
         }
-        float y = 0.0f;
+        float y[2] = {0.0f, 0.0f};
+        int stop = 0;
 #pragma unroll 1
         for (int layer = 0; layer < 3; ++layer) {
+            // the block meets once per layer, with every operand row written; a wait that gave up
+            // in an earlier layer ends the loop for all
             fence_async_smem();
             tc_fence_before();
-            __syncthreads();
+            stop = __syncthreads_or(late);
+            if (stop) break;
             if (tid == 0) {
                 tc_fence_after();
                 const uint32_t bw = layer == 0 ? SM_B2 : (layer == 1 ? SM_B3 : SM_B4);
                 const uint32_t idesc = layer == 2 ? IDESC4 : IDESC;
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    mma_k16(taddr, smem_desc(sbase + SM_A + 256 * kk), smem_desc(sbase + bw + 256 * kk), kk > 0,
-                            idesc);
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_k16(taddr + 64 * h, smem_desc(sbase + SM_A + h * (SM_A1 - SM_A) + 256 * kk),
+                                smem_desc(sbase + bw + 256 * kk), kk > 0, idesc);
                 mma_commit(&mbar);
             }
-            pending = 1;
-            if (!mbar_wait_bounded(&mbar, phase)) s_err = 1;
-            __syncthreads();
-            if (s_err) break;
-            pending = 0;
+            // each thread goes on when the group has completed; the next group needs all of them
+            if (!mbar_wait_bounded(&mbar, phase)) late = 1;
             phase ^= 1;
             tc_fence_after();
-            // layers 2 and 3: the SiLU row goes to A (the MMA that read A has completed); the
+            // layers 2 and 3: the SiLU rows go to A (the MMAs that read A have completed); the
             // output layer: column 0 plus b4
-            if (layer < 2) epilogue(t_row, layer == 0 ? hb2 : hb3, sm + SM_A, tid);
-            else y = tmem_ld1(t_row) + *b4;
+            if (layer < 2) {
+                epilogue(t_row, layer == 0 ? hb2 : hb3, sm + SM_A, tid);
+            } else {
+                y[0] = tmem_ld1(t_row) + *b4;
+                y[1] = tmem_ld1(t_row + 64) + *b4;
+            }
             tc_fence_before();
         }
-        if (s_err) break;
-        float xi_v = 0.0f, xc_v = 0.0f;
-        if (valid) {
-            float xi, xc;
-            if (bad) {
-                ++n_nan;
-                xi = 0.0f;
-                xc = 0.0f;
-            } else if (a.K.pair) {
-                bool oor = false;
-                if (fallback) {
-                    pair_shares<float>(a.inv, chi, r, xi, xc, oor);
-                    n_oor += oor;
-                    ++n_fb;
-                } else {
-                    // 1 - v-bar = exp(-u e^y): at most 1 for any network output
-                    const float small = 0.5f * expf(-expf(y + logf(u))), big = 1.0f - small;
-                    xi = rp >= 0.0f ? big : small;
-                    xc = rp >= 0.0f ? small : big;
-                }
-            } else {
-                float s;
-                if (fallback) {
+        if (stop) break;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t i = tile * IS + h * IT + tid;
+            const bool valid = i < n_all;
+            float xi_v = 0.0f, xc_v = 0.0f;
+            if (valid) {
+                float xi, xc;
+                if (bad[h]) {
+                    ++n_nan;
+                    xi = 0.0f;
+                    xc = 0.0f;
+                } else if (a.K.pair) {
                     bool oor = false;
-                    s = photon_s<float>(a.inv, chi, u, oor);
-                    n_oor += oor;
-                    ++n_fb;
+                    if (fallback[h]) {
+                        pair_shares<float>(a.inv, chi[h], r[h], xi, xc, oor);
+                        n_oor += oor;
+                        ++n_fb;
+                    } else {
+                        // 1 - v-bar = exp(-u e^y): at most 1 for any network output
+                        const float small = 0.5f * expf(-expf(y[h] + logf(u[h]))), big = 1.0f - small;
+                        const bool pos = 2.0f * r[h] - 1.0f >= 0.0f;
+                        xi = pos ? big : small;
+                        xc = pos ? small : big;
+                    }
                 } else {
-                    s = 1.5f * chi * expf(3.0f * (y + logf(u)));
+                    float s;
+                    if (fallback[h]) {
+                        bool oor = false;
+                        s = photon_s<float>(a.inv, chi[h], u[h], oor);
+                        n_oor += oor;
+                        ++n_fb;
+                    } else {
+                        s = 1.5f * chi[h] * expf(3.0f * (y[h] + logf(u[h])));
+                    }
+                    xc = 1.0f / (1.0f + s);
+                    xi = s < 1e30f ? s * xc : 1.0f;
                 }
-                xc = 1.0f / (1.0f + s);
-                xi = s < 1e30f ? s * xc : 1.0f;
+                a.xi[i] = xi;
+                if (a.xi_c) a.xi_c[i] = xc;
+                xi_v = xi;
+                xc_v = xc;
             }
-            a.xi[i] = xi;
-            if (a.xi_c) a.xi_c[i] = xc;
-            xi_v = xi;
-            xc_v = xc;
-        }
-        if (APPLY) {
-            // recoil of the emitter and the photon's record (every lane takes part in the
-            // warp-wide reservation)
-            const ApplyOut &o = a.ap;
-            const bool emit = valid && !bad;
-            const unsigned long long slot = warp_reserve(o.ocount, emit);
-            if (emit) {
-                // xi and 1 - xi = 1/(1 + s), the latter with relative precision (hard photons)
-                const float xi = xi_v, xc = xc_v;
-                const int64_t e = o.idx[i];
-                const float g = o.g[i], px = o.px[i], py = o.py[i], pz = o.pz[i];
-                const float pm = sqrtf(fmaf(px, px, fmaf(py, py, pz * pz)));
-                const float inv_pm = pm > 0.0f ? 1.0f / pm : 0.0f;
-                const float nx = px * inv_pm, ny = py * inv_pm, nz = pz * inv_pm;
-                const float gph = g * xi, gnew = g * xc;
-                const float q2 = fmaf(gnew, gnew, -1.0f);
-                const float pnew = q2 > 0.0f ? sqrtf(q2) : 0.0f;
-                n_g1 += !(q2 > 0.0f);
-                const uint8_t fl = o.flags[e];
-                if (slot < (unsigned long long)o.cap) {
-                    o.opx[slot] = nx * gph; o.opy[slot] = ny * gph; o.opz[slot] = nz * gph;
-                    o.opid[slot] = o.id ? o.id[e] : o.id_base + (uint64_t)e;
-                    o.ostep[slot] = o.step;
-                    o.ometa[slot] = (uint8_t)(SFQ_PHOTON | (((fl >> SFQ_TAG_SHIFT) & 3u) << 4));
-                } else {
-                    ++n_drop;
+            if (APPLY) {
+                // recoil of the emitter and the photon's record (every lane takes part in the
+                // warp-wide reservation)
+                const ApplyOut &o = a.ap;
+                const bool emit = valid && !bad[h];
+                const unsigned long long slot = warp_reserve(o.ocount, emit);
+                if (emit) {
+                    // xi and 1 - xi = 1/(1 + s), the latter with relative precision (hard photons)
+                    const float xi = xi_v, xc = xc_v;
+                    const int64_t e = o.idx[i];
+                    const float g = o.g[i], px = o.px[i], py = o.py[i], pz = o.pz[i];
+                    const float pm = sqrtf(fmaf(px, px, fmaf(py, py, pz * pz)));
+                    const float inv_pm = pm > 0.0f ? 1.0f / pm : 0.0f;
+                    const float nx = px * inv_pm, ny = py * inv_pm, nz = pz * inv_pm;
+                    const float gph = g * xi, gnew = g * xc;
+                    const float q2 = fmaf(gnew, gnew, -1.0f);
+                    const float pnew = q2 > 0.0f ? sqrtf(q2) : 0.0f;
+                    n_g1 += !(q2 > 0.0f);
+                    const uint8_t fl = o.flags[e];
+                    if (slot < (unsigned long long)o.cap) {
+                        o.opx[slot] = nx * gph; o.opy[slot] = ny * gph; o.opz[slot] = nz * gph;
+                        o.opid[slot] = o.id ? o.id[e] : o.id_base + (uint64_t)e;
+                        o.ostep[slot] = o.step;
+                        o.ometa[slot] = (uint8_t)(SFQ_PHOTON | (((fl >> SFQ_TAG_SHIFT) & 3u) << 4));
+                    } else {
+                        ++n_drop;
+                    }
+                    o.ppx[e] = nx * pnew; o.ppy[e] = ny * pnew; o.ppz[e] = nz * pnew;
+                    // a lepton left without momentum leaves the step (as in the step kernels)
+                    if (!(pnew > 0.0f)) o.flags[e] = (uint8_t)(fl & ~SFQ_ALIVE);
+                    ++n_emit;
                 }
-                o.ppx[e] = nx * pnew; o.ppy[e] = ny * pnew; o.ppz[e] = nz * pnew;
-                // a lepton left without momentum leaves the step (as in the step kernels)
-                if (!(pnew > 0.0f)) o.flags[e] = (uint8_t)(fl & ~SFQ_ALIVE);
-                ++n_emit;
             }
         }
     }
     // a group whose wait gave up: wait once more (bounded) before the tensor memory is freed
-    if (pending && tid == 0) {
-        if (!mbar_wait_bounded(&mbar, phase) && a.status) atomicExch(a.status, 1);
+    const int failed = __syncthreads_or(late);
+    if (failed && tid == 0) {
+        if (!mbar_wait_bounded(&mbar, phase ^ 1) && a.status) atomicExch(a.status, 1);
     }
-    if (s_err && tid == 0 && a.counters) atomicAdd(&a.counters->timeouts, 1ull);
+    if (failed && tid == 0 && a.counters) atomicAdd(&a.counters->timeouts, 1ull);
     atomicAdd(&s_cnt[0], (unsigned long long)n_nan);
     atomicAdd(&s_cnt[1], (unsigned long long)n_oor);
     atomicAdd(&s_cnt[2], (unsigned long long)n_fb);
@@ -758,7 +815,7 @@ __global__ void __launch_bounds__(IT, INFER_MINB) infer_tc_kernel(const InferArg
             if (s_cnt[5]) atomicAdd(&a.counters->gamma_below_one, s_cnt[5]);
         }
     }
-    if (s_err && tid == 0 && a.status) atomicExch(a.status, 1);
+    if (failed && tid == 0 && a.status) atomicExch(a.status, 1);
 }
 
 }  // namespace mlp
@@ -771,7 +828,7 @@ cudaError_t launch_surrogate_apply(const sfq_ctx *ctx, const sfq_particles *p, u
     const sfq_mlp *m = ctx->surr;
     const sfq_event_queue &q = ctx->surr_q;
     if (q.capacity <= 0) return cudaSuccess;
-    const int64_t ntiles = (q.capacity + IT - 1) / IT;
+    const int64_t ntiles = (q.capacity + IS - 1) / IS;
     int64_t grid = (int64_t)ctx->surr_per_sm * ctx->num_sms;
     if (ntiles < grid) grid = ntiles;
     InferArgs a{};
@@ -836,9 +893,9 @@ struct DeviceGuard {
 bool a16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Attributes of an inference kernel instance: its dynamic shared memory, and the largest
-// shared-memory carveout, so that INFER_MINB blocks (6 x 36 KB) are resident on an SM.  The
-// grid is then INFER_MINB blocks per SM: registers (at most 85 a thread by the launch
-// bounds), shared memory and tensor memory (6 x 64 of the 512 columns) all admit them.
+// shared-memory carveout, so that INFER_MINB blocks (4 x 53 KB) are resident on an SM.  The
+// grid is then INFER_MINB blocks per SM: registers (at most 128 a thread by the launch
+// bounds), shared memory and tensor memory (4 x 128 of the 512 columns) all admit them.
 template <typename K>
 cudaError_t set_infer_attributes(K kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)INFER_SMEM);
@@ -1057,7 +1114,7 @@ static sfq_status mlp_sample(sfq_mlp *m, int64_t n, const void *chi, const void 
         attr = true;
     }
     const int per_sm = INFER_MINB;
-    const int64_t ntiles = (n + IT - 1) / IT;
+    const int64_t ntiles = (n + IS - 1) / IS;
     int64_t grid = (int64_t)per_sm * m->ctx->num_sms;
     if (ntiles < grid) grid = ntiles;
     InferArgs a{m->params, use_flags ? m->flags : nullptr, inv_table(m), n,

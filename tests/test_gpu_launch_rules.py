@@ -157,3 +157,26 @@ def test_loss_and_gradient_around_the_reduction_chunks(n):
     ref.backward()
     assert abs(float(loss) / float(ref.detach()) - 1) < 1.5e-5
     assert float((grad.double() - th.grad).norm() / th.grad.norm()) < 1.5e-5
+
+
+@pytest.mark.parametrize("kind", ["photon", "pair"])
+def test_surrogate_tiles(kind):
+    """The tensor-core kernel takes tiles of 256 draws, two per thread: calls around a tile and
+    around one wave of blocks give the draws of a longer call, with and without the flags."""
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision="fp32", seed=4)
+    net = sfq.Surrogate(ctx, seed=3, kind=kind)
+    net.calibrate(0.2)                                          # an untrained network: some cells flagged, not all
+    wave = torch.cuda.get_device_properties(0).multi_processor_count * 4 * 256
+    big = 2 * wave + 300
+    _, chi, r = _elements(big, torch.float32)
+    sample = net.sample_photon_xi if kind == "photon" else net.sample_pair_xi
+    for flags in (False, True):
+        cnt = [sfq.counters_tensor() for _ in range(2)]
+        whole = sample(chi, r, use_flags=flags, counters=cnt[0])
+        for n in (1, 127, 128, 129, 255, 256, 257, 511, wave - 1, wave, wave + 1):
+            for a, b in zip(sample(chi[:n], r[:n], use_flags=flags), whole):
+                assert torch.equal(a.view(torch.int32), b[:n].view(torch.int32)), n
+        for k in range(0, big, 70144):
+            sample(chi[k:k + 70144], r[k:k + 70144], use_flags=flags, counters=cnt[1])
+        assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
+        assert (sfq.counters_dict(cnt[0])["surrogate_fallbacks"] > 0)
