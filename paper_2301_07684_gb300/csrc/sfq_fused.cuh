@@ -7,8 +7,11 @@
 // B = (0, 0, a C), C = cos table[(k0 + step k_step) mod K], nothing has to leave the SM
 // between steps: this kernel loads a particle once, runs steps step0 ... step0+nsteps-1
 // on it and stores it once.  The arithmetic of every update and of every event is the
-// per-step kernels' own (step_particle_v with the plane-wave chi, process_events_core),
-// so the records, final states and counters equal those of nsteps sfq_mc_step calls.
+// per-step kernels' own (step_pair and step_particle_v with the plane-wave chi,
+// process_events_core), so the records, final states and counters equal those of nsteps
+// sfq_mc_step calls.  Issue bounds it: 100 steps of 2^20 particles took 1595 us slot by slot
+// (55 % of the issue slots, 23.7 of 32 lanes active), 1337 us with two slots of a lane in
+// packed registers (62 %, 28.9 lanes).
 //
 // Each lane holds PPL particles ("slots"), each with its own step counter.  An update
 // that ends in an event puts the slot on the warp's event queue and the slot waits; the
@@ -101,27 +104,62 @@ __global__ void __launch_bounds__(FUSED_BS, 2) mc_fused_kernel(const StepArgs<T>
         unsigned qt = 0, qh = 0;               // warp-uniform queue tail and head
         for (;;) {
             bool ran = false;
+            bool evs[PPL];
+            T gs[PPL], cs[PPL];
 #pragma unroll
-            for (int k = 0; k < PPL; ++k) {
-                const int64_t i = base + k * 32 + lane;
-                const bool run = in[k] && (fl[k] & SFQ_ALIVE) && !pend[k] && st[k] < nsteps;
-                bool ev = false;
-                T g = (T)0, chi = (T)0;
-                if (run) {
-                    ran = true;
+            for (int k0s = 0; k0s < PPL; k0s += 2) {
+                // two slots at a time: binary32 leptons in packed registers (step_pair), a slot that
+                // does not run masked; other species and binary64 one by one
+                bool run[2], photon = false;
+                T f[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int k = k0s + j;
+                    run[j] = in[k] && (fl[k] & SFQ_ALIVE) && !pend[k] && st[k] < nsteps;
+                    ran |= run[j];
+                    photon |= run[j] && ((fl[k] >> SFQ_SPECIES_SHIFT) & 3u) == SFQ_PHOTON;
                     uint32_t kk = k0[k] + off[k];               // as the per-step field source
                     kk -= (kk >= K) ? K : 0u;
                     kk = kk < K ? kk : K - 1u;
-                    const T f = amp[k] * s_tab[kk];
-                    const T E[3] = {(T)0, f, (T)0}, B[3] = {(T)0, (T)0, f};
-                    ev = step_particle_v<T, true>(a, s_nlc, s_nbw, i, (uint8_t)fl[k], px[k], py[k], pz[k], E, B,
-                                                  tau[k], g, chi, c, step0 + st[k]);
-                    if (!ev) {
-                        ++st[k];
-                        off[k] += kstep;
-                        off[k] -= (off[k] >= K) ? K : 0u;
+                    f[j] = amp[k] * s_tab[kk];
+                    evs[k] = false;
+                    gs[k] = cs[k] = (T)0;
+                }
+                if (sizeof(T) == 4 && !photon) {
+                    if constexpr (sizeof(T) == 4) {
+                        const auto two = [](const T *v) { return f32x2(v[0], v[1]); };
+                        const f32x2 E[3] = {f32x2(0ull), two(f), f32x2(0ull)};
+                        const auto fill = [&](int j, uint64_t bits) {
+                            const int64_t i = base + (k0s + j) * 32 + lane;
+                            const auto id_of = [&]() { return a.id ? a.id[i] : a.id_base + (uint64_t)i; };
+                            return od_fill(bits, a.seed, id_of, step0 + st[k0s + j], (fl[k0s + j] >> SFQ_TAG_SHIFT) & 3u);
+                        };
+                        step_pair<true, false, true>(a, s_nlc, run, fill, two(px + k0s), two(py + k0s), two(pz + k0s), E, E,
+                                                     tau + k0s, gs + k0s, cs + k0s, evs + k0s, c);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const int k = k0s + j;
+                        if (!run[j]) continue;
+                        const T E[3] = {(T)0, f[j], (T)0}, B[3] = {(T)0, (T)0, f[j]};
+                        evs[k] = step_particle_v<T, true>(a, s_nlc, s_nbw, base + k * 32 + lane, (uint8_t)fl[k], px[k], py[k],
+                                                          pz[k], E, B, tau[k], gs[k], cs[k], c, step0 + st[k]);
                     }
                 }
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    if (run[j] && !evs[k0s + j]) {
+                        ++st[k0s + j];
+                        off[k0s + j] += kstep;
+                        off[k0s + j] -= (off[k0s + j] >= K) ? K : 0u;
+                    }
+            }
+#pragma unroll
+            for (int k = 0; k < PPL; ++k) {
+                const int64_t i = base + k * 32 + lane;
+                const bool ev = evs[k];
+                const T g = gs[k], chi = cs[k];
                 const unsigned m = __ballot_sync(0xFFFFFFFFu, ev);
                 if (ev) {
                     const unsigned r = qt + __popc(m & ((1u << lane) - 1u));

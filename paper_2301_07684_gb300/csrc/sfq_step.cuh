@@ -649,19 +649,19 @@ __device__ __forceinline__ float wtilde_pair_sel(const float *c, float chi, bool
 // that a population's warps stay in one path (with a block for two alive photons only, warps
 // ran it and the general path: 31 us against 27 for 1e6 photons of which a third has
 // converted).  Leptons rarely do, and the mask cost them 3 % of a plane-wave step.
-// E[1] alone is read with the plane wave; tab is the species' rate table.
-template <bool PW, bool PHOTON>
-__device__ __forceinline__ void step_pair(const StepArgs<float> &a, const float *tab, int64_t i0, uint32_t fl2,
+// E[1] alone is read with the plane wave; tab is the species' rate table; act: which of the
+// two are stepped (read when MASK); fill(k, bits): the optical depth particle k starts from
+// (od_fill).
+template <bool PW, bool PHOTON, bool MASK, typename Fill>
+__device__ __forceinline__ void step_pair(const StepArgs<float> &a, const float *tab, const bool act[2], Fill fill,
                                           f32x2 px, f32x2 py, f32x2 pz, const f32x2 E[3], const f32x2 B[3],
                                           double tau[2], float g[2], float chi[2], bool ev[2], Cnt &c) {
-    const bool on[2] = {!PHOTON || (fl2 & SFQ_ALIVE) != 0u, !PHOTON || (fl2 & (SFQ_ALIVE << 8)) != 0u};
+    const bool on[2] = {!MASK || act[0], !MASK || act[1]};
     uint64_t b[2] = {(uint64_t)__double_as_longlong(tau[0]), (uint64_t)__double_as_longlong(tau[1])};
-    if (PHOTON ? (on[0] && (int64_t)b[0] < 0) || (on[1] && (int64_t)b[1] < 0) : (int64_t)(b[0] | b[1]) < 0) {
+    if (MASK ? (on[0] && (int64_t)b[0] < 0) || (on[1] && (int64_t)b[1] < 0) : (int64_t)(b[0] | b[1]) < 0) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const auto id_of = [&]() { return a.id ? a.id[i0 + k] : a.id_base + (uint64_t)(i0 + k); };
-            if (on[k]) b[k] = od_fill(b[k], a.seed, id_of, a.step, (fl2 >> (8 * k + SFQ_TAG_SHIFT)) & 3u);
-        }
+        for (int k = 0; k < 2; ++k)
+            if (on[k]) b[k] = fill(k, b[k]);
     }
     const f32x2 one(1.0f, 1.0f), half(0.5f, 0.5f);
     const f32x2 p2 = fma2(px, px, fma2(py, py, mul2(pz, pz)));

@@ -313,13 +313,19 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
             constexpr uint32_t AL = SFQ_ALIVE * 0x0101u, SP = 3u << SFQ_SPECIES_SHIFT,
                                PH = (SFQ_PHOTON << SFQ_SPECIES_SHIFT) * 0x0101u;
             const uint32_t sx = vf ^ PH;                   // a zero species field: photon
+            const bool on[2] = {(vf & SFQ_ALIVE) != 0u, (vf & (SFQ_ALIVE << 8)) != 0u};
+            const auto fill = [&](int k, uint64_t bits) {
+                const int64_t i = start + li0 + k;
+                const auto id_of = [&]() { return a.id ? a.id[i] : a.id_base + (uint64_t)i; };
+                return od_fill(bits, a.seed, id_of, a.step, (vf >> (8 * k + SFQ_TAG_SHIFT)) & 3u);
+            };
             const bool lep0 = (vf & SFQ_ALIVE) && (sx & SP), lep1 = (vf & (SFQ_ALIVE << 8)) && (sx & (SP << 8));
             if ((vf & AL) == AL && (sx & SP) && (sx & (SP << 8))) {
                 if constexpr (PAIRED)
-                    step_pair<FK == FK_PW, false>(a, s_nlc, start + li0, vf, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
+                    step_pair<FK == FK_PW, false, false>(a, s_nlc, on, fill, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
             } else if (!lep0 && !lep1) {
                 if constexpr (PAIRED)
-                    step_pair<FK == FK_PW, true>(a, s_nbw, start + li0, vf, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
+                    step_pair<FK == FK_PW, true, true>(a, s_nbw, on, fill, vx, vy, vz, E2, B2, tau_out, gk, ck, ev, c);
             } else if constexpr (PAIRED) {
                 T e2[3][2], b2[3][2];
 #pragma unroll
