@@ -366,11 +366,9 @@ sfq_status sfq_cascade_run(sfq_ctx *ctx, const sfq_particles *p, const sfq_field
     DeviceGuard g(ctx->device);
     const cudaStream_t s = (cudaStream_t)stream;
     unsigned long long *count = const_cast<unsigned long long *>(p->n_dev);
-    cudaError_t e = sfq::launch_cascade_sync(count, next, p->n, true, s);
-    for (uint32_t j = 0; j < nsteps && e == cudaSuccess; ++j) {
+    cudaError_t e = sfq::launch_cascade_begin(count, next, p->n, s);
+    for (uint32_t j = 0; j < nsteps && e == cudaSuccess; ++j)
         e = sfq::launch_step(ctx, p, f, step0 + j, out, &sp, counters, s, 1);
-        if (e == cudaSuccess) e = sfq::launch_cascade_sync(count, next, p->n, false, s);
-    }
     return e == cudaSuccess ? SFQ_OK : cuda_fail(ctx, e, "sfq_cascade_run");
 }
 

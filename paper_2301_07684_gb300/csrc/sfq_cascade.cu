@@ -1,4 +1,4 @@
-// sfq_cascade.cu -- device side of the full cascade: the count commit between steps and the
+// sfq_cascade.cu -- device side of the full cascade: the start of a run's count and the
 // stable stream compaction of a population (count, scan, scatter into a second buffer set).
 #include <cstdint>
 
@@ -12,16 +12,12 @@ constexpr int CG_PER_SM = 8;         // compaction blocks per SM (the grid)
 constexpr int CG_MAX = 4096;         // largest compaction grid (bounds the scratch)
 constexpr int SCAN_BS = 1024;        // the single block of the scan
 
-// begin: clamp the live count to the capacity and start the append counter there; after a
-// step: the appended total (clamped) becomes the live count of the next step.
-__global__ void cascade_sync_kernel(unsigned long long *count, unsigned long long *next, unsigned long long cap,
-                                    int begin) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        unsigned long long c = begin ? *count : *next;
-        c = c < cap ? c : cap;
-        *count = c;
-        *next = c;
-    }
+// Before a run: clamp the live count to the capacity and start the append counter there (each
+// step's kernel commits its own appended total: cascade_commit).
+__global__ void cascade_begin_kernel(unsigned long long *count, unsigned long long *next, unsigned long long cap) {
+    const unsigned long long c = *count < cap ? *count : cap;
+    *count = c;
+    *next = c;
 }
 
 __device__ __forceinline__ int64_t live_count(const unsigned long long *count, int64_t n) {
@@ -222,9 +218,8 @@ cudaError_t compact_t(const sfq_particles &src, const sfq_fields &fsrc, const sf
 
 }  // namespace
 
-cudaError_t launch_cascade_sync(unsigned long long *count, unsigned long long *next, int64_t cap, bool begin,
-                                cudaStream_t s) {
-    cascade_sync_kernel<<<1, 32, 0, s>>>(count, next, (unsigned long long)cap, begin ? 1 : 0);
+cudaError_t launch_cascade_begin(unsigned long long *count, unsigned long long *next, int64_t cap, cudaStream_t s) {
+    cascade_begin_kernel<<<1, 1, 0, s>>>(count, next, (unsigned long long)cap);
     return cudaGetLastError();
 }
 

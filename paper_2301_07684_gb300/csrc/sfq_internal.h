@@ -110,9 +110,8 @@ sfq_status validate_step(sfq_ctx *ctx, const sfq_particles *p, const sfq_fields 
 cudaError_t launch_step(const sfq_ctx *ctx, const sfq_particles *p, const sfq_fields *f, uint32_t step,
                         const sfq_products *out, const sfq_spawn *spawn, sfq_counters *counters, cudaStream_t stream,
                         int cascade = 0);
-// Full cascade (sfq_cascade.cu): the count commit around a step and the stream compaction.
-cudaError_t launch_cascade_sync(unsigned long long *count, unsigned long long *next, int64_t cap, bool begin,
-                                cudaStream_t s);
+// Full cascade (sfq_cascade.cu): the start of a run's append counter, and the stream compaction.
+cudaError_t launch_cascade_begin(unsigned long long *count, unsigned long long *next, int64_t cap, cudaStream_t s);
 size_t compact_scratch_bytes(int64_t capacity);
 cudaError_t launch_compact(int precision, const sfq_particles &src, const sfq_fields &fsrc, const sfq_particles &dst,
                            const sfq_fields &fdst, void *scratch, cudaStream_t s, int num_sms);

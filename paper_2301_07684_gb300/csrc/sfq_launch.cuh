@@ -290,6 +290,7 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
         const int64_t need = (chunks + STEP_BS / 32 - 1) / (STEP_BS / 32);
         if (need < grid) grid = (int)(need > 0 ? need : 1);
     }
+    if (L.cascade && grid > 65535) grid = 65535;       // the commit counts blocks in 16 bits
     kern<<<grid, STEP_BS, 0, L.stream>>>(a);
     return cudaGetLastError();
 }
