@@ -95,7 +95,7 @@ static cudaError_t launch_uniforms_t(int64_t n, const uint64_t *id, uint32_t ste
 // The TMA-staged shapes compiled with the truncated samplers (TRUNC) are limited to 16
 // consumer warps; the warp-streaming ones to 2 particles per lane.
 constexpr int TRUNC_CW = 16, TRUNC_PPT = 2;
-// Consumer warps per block of the default shape.  With the producer they are 20 or 16 warps, 5
+// Consumer warps per block of the default binary32 shapes.  With the producer they are 20 or 16 warps, 5
 // or 4 per scheduler, which leaves 96 or 128 registers a thread (16 consumer warps: 17, five
 // on one scheduler).  Fields in memory wait on HBM and on event batches, where more warps
 // help: 8 steps of 2^24 particles 1539 us with 19, 1552 with 15, 1574 with 23 (80 registers).
@@ -121,9 +121,12 @@ static cudaError_t prepare_step_t() {
         SFQ_PREP(8)
         SFQ_PREP(16)
         SFQ_PREP(20)
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>());
+        if constexpr (sizeof(T) == 4) {
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>());
+        }
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_PW, TMA_CW_PW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tma_smem_bytes<T, FK_PW, TMA_CW_PW>());
@@ -213,13 +216,25 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
     if (p.n == 0) return cudaSuccess;
     const StepArgs<T> a = make_step_args<T>(L);
     const bool pw = f.kind == SFQ_FIELDS_PLANE_WAVE;
-    // TMA-staged kernel: one persistent block per SM; chosen automatically when every
-    // SM gets at least one full tile.  `ppt` selects the consumer warps per block.
-    const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : (pw ? TMA_CW_PW : TMA_CW_SOA));
-    const int tile = (cw < 16 ? cw : 16) * (sizeof(T) == 4 ? 64 : 32);
+    // TMA-staged kernel: one persistent block per SM; `ppt` selects the consumer warps per block.
+    // Chosen automatically (us per step in a graph, warp-streaming against TMA-staged):
+    //  - binary32, fields in memory: from ten tiles per SM, where the pipeline has filled (150,000
+    //    particles 10.9 / 12.5, 300,000 13.6 / 16.3, 10^6 19.4 / 20.8, 2*10^6 33.2 / 29.3);
+    //  - binary32, plane wave: from a tile per SM (11.1 / 11.9 at 150,000, 13.8 / 13.6 at 300,000,
+    //    31.6 / 30.6 at 2*10^6);
+    //  - binary64: from 128 particles per SM (28 / 27 at 20,000, 80 / 44 at 160,000, 556 / 532 at
+    //    4*10^6), with 8 consumer warps: the FP64 pipe takes two lanes per clock and SM whatever
+    //    a warp's active lanes, 8 warps keep it busy and leave 8 partial event batches at the
+    //    end instead of 16 (62) or 19 (67 us at 160,000).  Only a plane wave of millions of
+    //    particles gains from more (507 / 493 us at 4*10^6).
+    const bool f64 = sizeof(T) == 8;
+    const int dflt = f64 ? (pw && p.n >= (1ll << 21) ? TMA_CW_PW : 8) : (pw ? TMA_CW_PW : TMA_CW_SOA);
+    const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : dflt);
+    const int tile = (cw < 16 ? cw : 16) * (f64 ? 32 : 64);
+    const int64_t tma_from = (int64_t)(TRUNC ? tile : (f64 ? 128 : (pw ? 1024 : 10 * 1024))) * ctx->num_sms;
     // the beyond-LCFA model runs on the warp-streaming kernel (its state is read directly)
     const bool tma = !L.cascade && p.lepton_model == SFQ_LEPTON_LCFA_OD &&
-                     (L.variant == 2 || (L.variant == 0 && p.n >= (int64_t)tile * ctx->num_sms));
+                     (L.variant == 2 || (L.variant == 0 && p.n >= tma_from));
     if (tma) {
         void (*kern)(const StepArgs<T>) = nullptr;
         size_t smem = 0;
@@ -243,8 +258,10 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
                     smem = tma_smem_bytes<T, FK_PW, TMA_CW_PW>();
                     break;
                 default:
-                    kern = mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>;
-                    smem = tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>();
+                    if constexpr (sizeof(T) == 4) {
+                        kern = mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>;
+                        smem = tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>();
+                    }
                     break;
             }
         }
