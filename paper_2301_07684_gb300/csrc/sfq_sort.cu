@@ -573,11 +573,17 @@ cudaError_t small_sort(const sfq_products &out, int n, cudaStream_t s) {
 cudaError_t sort_products(const sfq_products &out, int64_t n, size_t elem, void *scratch, cudaStream_t s,
                           int num_sms) {
     if (n <= 1) return cudaSuccess;
+    // a sort reads back key bits, so it is not recorded into a graph; the one-block sort would be,
+    // with its record count fixed, and is refused alike
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
     if (n <= SMALL_N) return elem == 4 ? small_sort<float>(out, (int)n, s) : small_sort<double>(out, (int)n, s);
     const Plan P = plan(n);
     char *sc = static_cast<char *>(scratch);
     Bits *bits = reinterpret_cast<Bits *>(sc + P.o_bits);
-    cudaError_t e = cudaMemsetAsync(bits, 0, sizeof(Bits), s);
+    e = cudaMemsetAsync(bits, 0, sizeof(Bits), s);
     if (e != cudaSuccess) return e;
     const int64_t blocks = (n + 256 * 8 - 1) / (256 * 8);
     bits_kernel<<<(unsigned)(blocks < num_sms * 8ll ? blocks : num_sms * 8ll), 256, 0, s>>>(n, out.parent_id, out.step,
