@@ -194,15 +194,17 @@ __device__ __forceinline__ int pair_piece(T chi, T a, T &xc, T &xr, bool &oor) {
 }
 
 // s = 3 chi w^3 / 2 for w-bar = G~_pe(r, chi) (Eq. again, Eq. subs_altri).  TR > 0 reads the
-// table truncated by TR degrees in each variable.
-template <typename T, int TR = 0, bool CH = false>
+// table truncated by TR degrees in each variable; AHEAD: horner2_ahead.
+template <typename T, int TR = 0, bool CH = false, bool AHEAD = false>
 __device__ __forceinline__ T photon_s(const T *__restrict__ inv, T chi, T r, bool &oor) {
     using Q = L<T>;
     constexpr int DX = Q::PI_DX - TR, DY = Q::PI_DY - TR;
     T xc, xr;
     bool low;
     const T *c = inv + (size_t)photon_piece<T>(chi, r, xc, xr, low, oor) * ((DX + 1) * padded_row(DY + 1, sizeof(T)));
-    T w = CH ? clenshaw2<DX, DY>(c, xc, xr) : horner2<DX, DY>(c, xc, xr);
+    T w;
+    if constexpr (AHEAD) w = horner2_ahead<DX, DY>(c, xc, xr);
+    else w = CH ? clenshaw2<DX, DY>(c, xc, xr) : horner2<DX, DY>(c, xc, xr);
     if (low) w *= r;                          // the low-r block holds w-bar / r
     const T chi_eff = chi > (T)4096 ? (T)4096 : chi;
     return (T)1.5 * chi_eff * w * w * w;
@@ -233,13 +235,13 @@ __device__ __forceinline__ void pair_shares(const T *__restrict__ inv, T chi, T 
 // full tables.  TRUNC = true reads the tables truncated by t.tr = 1 or 2 degrees in each
 // variable.  Kernels are instantiated with TRUNC = true only for contexts that use the
 // knob, so the default kernels carry no code for it.
-template <typename T, bool TRUNC>
+template <typename T, bool TRUNC, bool AHEAD = false>
 __device__ __forceinline__ T photon_s_sel(const Tables<T> &t, T chi, T r, bool &oor) {
     if (TRUNC) {
         if (t.tr == 2) return photon_s<T, 2>(t.nlc_inv_r, chi, r, oor);
         return photon_s<T, 1>(t.nlc_inv_r, chi, r, oor);
     }
-    return photon_s<T, 0>(t.nlc_inv, chi, r, oor);
+    return photon_s<T, 0, false, AHEAD && sizeof(T) == 4>(t.nlc_inv, chi, r, oor);
 }
 template <typename T, bool TRUNC>
 __device__ __forceinline__ void pair_shares_sel(const Tables<T> &t, T chi, T r, T &xe, T &xp, bool &oor) {

@@ -381,8 +381,9 @@ __device__ __forceinline__ void reserve_single(unsigned long long *ocount, unsig
 // global atomic per batch, before the sampling when every record count is known up
 // front (no beyond-LCFA lane, whose emission may be rejected), so that the atomic's
 // latency overlaps the sampling.
-// SINGLE: batches without a converted photon take the ballot reservation (the TMA-staged
-// kernel; the warp-streaming instances, held to 64 registers, lost 3 % to the extra code).
+// SINGLE: batches without a converted photon take the ballot reservation, and a sample's
+// coefficients are fetched ahead (the TMA-staged kernel; the warp-streaming instances, held
+// to 64 registers, lost 3 % to the extra code).
 template <typename T, bool TRUNC = false, bool CASC = false, bool SURR = false, bool SINGLE = false>
 __device__ __forceinline__ void process_events_core(const StepArgs<T> &a, uint32_t step, int64_t ei, T eg, T echi,
                                                     T e_aux, T px, T py, T pz, uint8_t fl, bool valid, Cnt &c,
@@ -434,7 +435,7 @@ __device__ __forceinline__ void process_events_core(const StepArgs<T> &a, uint32
                 a.qg[qslot] = (float)eg;
                 a.qpx[qslot] = (float)px; a.qpy[qslot] = (float)py; a.qpz[qslot] = (float)pz;
             } else {
-                xa = photon_s_sel<T, TRUNC>(a.tab, echi, r1, oor);  // s
+                xa = photon_s_sel<T, TRUNC, SINGLE>(a.tab, echi, r1, oor);  // s
                 ++c.v[C_EMIT];
             }
         } else {
