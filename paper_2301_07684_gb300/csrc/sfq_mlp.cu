@@ -350,8 +350,8 @@ __global__ void __launch_bounds__(RB) reduce_kernel(const float *__restrict__ pa
 }
 
 // ---------------------------------------------------------------------------------------
-// Tensor-core inference.  One block of 128 threads handles tiles of 128 samples (one
-// sample per thread, one row of the 128 x 64 activation tile).  Layers 2 and 3 are
+// Tensor-core inference.  One block of 128 threads handles tiles of 256 samples (two per
+// thread, one row of each of two 128 x 64 activation operands).  Layers 2 and 3 are, for each,
 //   D[128 x 64] (fp32, tensor memory) = A[128 x 64] (bf16, smem) * W^T (W: 64 x 64 bf16, smem)
 // issued as four K = 16 steps of tcgen05.mma.kind::f16 by one thread; the output layer is
 // the same with a 16 x 64 W whose row 0 is w4 (column 0 of D is the output).  Operands use the

@@ -9,8 +9,8 @@
 // warp busy with its events delays no stage's release.  Each consumer warp queues its event particles, with the
 // state it read, in a ring of its own and samples them 32 at a time.
 // What bounds it (binary32): with fields in memory 53 B per particle from and to HBM, about
-// 59 with the 32-byte sectors of the momenta that events rewrite; 2^24 particles take 180 us,
-// 81 % of the copy bandwidth on those bytes.  The plane wave, and populations too small to
+// 59 with the 32-byte sectors of the momenta that events rewrite; 2^24 particles take 175 us
+// (190 with two scalar particles per lane), 83 % of the copy bandwidth on those bytes.  The plane wave, and populations too small to
 // fill the stages many times, are bound by issue: two leptons of a lane are stepped in
 // packed registers without branches (step_pair), 6.5 warp-instructions per particle
 // with its events (8.2 before, when 4.2e6 particles took 57 us under the profiler with fields
