@@ -230,7 +230,7 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
     const bool f64 = sizeof(T) == 8;
     const int dflt = f64 ? (pw && p.n >= (1ll << 21) ? TMA_CW_PW : 8) : (pw ? TMA_CW_PW : TMA_CW_SOA);
     const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : dflt);
-    const int tile = (cw < 16 ? cw : 16) * (f64 ? 32 : 64);
+    const int tile = cw * (f64 ? 32 : 64);
     const int64_t tma_from = (int64_t)(TRUNC ? tile : (f64 ? 128 : (pw ? 1024 : 10 * 1024))) * ctx->num_sms;
     // the beyond-LCFA model runs on the warp-streaming kernel (its state is read directly)
     const bool tma = !L.cascade && p.lepton_model == SFQ_LEPTON_LCFA_OD &&

@@ -4,10 +4,11 @@
 // slices (momenta, optical depth, flags, fields or phase index) from global to
 // shared memory with 1D bulk copies (cp.async.bulk), NSTAGE tiles ahead, and the
 // consumer warps compute the step (Sec. 2 and 4 of Montefiori & Tamburini,
-// arXiv:2301.07684) from shared memory.  A tile is cut into slices of 32 or 64 particles;
-// with fields in memory the warps claim the slices in order from a shared counter, so a
-// warp busy with its events delays no stage's release.  Each consumer warp queues its event particles, with the
-// state it read, in a ring of its own and samples them 32 at a time.
+// arXiv:2301.07684) from shared memory.  A tile is cut into slices of 32 or 64 particles, as
+// many as there are consumer warps; with fields in memory the warps claim the slices in order
+// from a shared counter, so a warp busy with its events delays no stage's release.  Each
+// consumer warp queues its event particles, with the state it read, in a ring of its own and
+// samples them 32 at a time.
 // What bounds it (binary32): with fields in memory 53 B per particle from and to HBM, about
 // 59 with the 32-byte sectors of the momenta that events rewrite; 2^24 particles take 175 us
 // (190 with two scalar particles per lane), 83 % of the copy bandwidth on those bytes.  The plane wave, and populations too small to
@@ -77,13 +78,12 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-// Layout of one stage: a tile of SLICES slices, each one warp's work (2 particles per lane in
-// binary32, 1 in binary64).  A block of up to 16 consumer warps has a slice per warp; more
-// warps share tiles of 16 slices, so that the stages leave room for their event queues.
+// Layout of one stage: a tile of one slice per consumer warp, 2 particles per lane in binary32,
+// 1 in binary64.  No fewer slices than warps: the stages' hand-over needs it (see the
+// consumers' loop).
 template <typename T, int FK, int CW>
 struct TmaStage {
-    static constexpr int SLICES = CW < 16 ? CW : 16;
-    static constexpr int TILE = SLICES * (sizeof(T) == 4 ? 64 : 32);
+    static constexpr int TILE = CW * (sizeof(T) == 4 ? 64 : 32);
     static constexpr int NF = FK == FK_SOA ? 6 : 0;
     static constexpr size_t O_PX = 0, O_PY = O_PX + TILE * sizeof(T), O_PZ = O_PY + TILE * sizeof(T);
     static constexpr size_t O_TAU = O_PZ + TILE * sizeof(T);
@@ -100,7 +100,7 @@ struct TmaStage {
 template <typename T, int FK, int CW>
 struct TmaCfg {
     using S = TmaStage<T, FK, CW>;
-    static constexpr int PPL = S::TILE / S::SLICES / 32;           // particles per lane per slice
+    static constexpr int PPL = S::TILE / CW / 32;                  // particles per lane per slice
     static constexpr int QS = 32 * (PPL + 1);                      // one slice's events plus a partial batch
     static constexpr size_t QBYTES = (size_t)CW * QS * sizeof(QEntry<T>);
     static constexpr size_t STATIC = (RateSmem<T>::NLC_N + RateSmem<T>::NBW_N) * sizeof(T);
@@ -145,8 +145,7 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     constexpr int TMA_CONSUMER_WARPS = CW;
     constexpr int TMA_THREADS = 32 * (CW + 1);
     constexpr int TILE = S::TILE;
-    constexpr int SLICES = S::SLICES;
-    constexpr int PER_WARP = TILE / SLICES;                // particles per slice
+    constexpr int PER_WARP = TILE / CW;                    // particles per slice
     constexpr int PPL = CFG::PPL;                          // particles per lane per slice
     constexpr int QS = CFG::QS;                            // one slice + a partial batch
     constexpr bool PAIRED = sizeof(T) == 4 && PPL == 2;     // adjacent-pair vector layout
@@ -168,7 +167,7 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     if (threadIdx.x == 0) {
         for (int s = 0; s < TMA_NSTAGE; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], SLICES);
+            mbar_init(&empty[s], CW);
         }
         *abort_flag = 0;
         *slice_ctr = 0;
@@ -240,20 +239,24 @@ __global__ void __launch_bounds__(32 * (CW + 1), 1) mc_step_tma_kernel(const Ste
     // With fields in memory (SoA) the step waits on HBM and on its events: a warp takes the
     // block's next slice (one warp's share, PER_WARP particles, of tile t) from a shared
     // counter, so a warp that is sampling its events leaves the next slices to the others
-    // instead of holding up the release of their stage.  Slices are claimed in order and each
-    // warp holds one claim, so no warp can wait on a stage two phases ahead: the slices of
-    // the NSTAGE tiles before that phase (at least 2 x 16) would all have to be held by
-    // warps waiting for them, besides the one that keeps the stage.  With the plane wave the
-    // step is bound by issue, and the warps take the slices in turn (no claim); a warp's next
-    // slice is then at most two tiles ahead of its last, and again less than two phases.
+    // instead of holding up the release of their stage.  With the plane wave a warp takes its
+    // own slice of every tile (no claim).
+    // A barrier's parity tells a phase from the next one only, so no warp may wait for tile t
+    // before tile t - NSTAGE, the phase before on the same stage, has landed; tiles may land
+    // in any order.  Slices are claimed in order and a warp holds one claim: when a slice of
+    // tile t is claimed, the CW slices of tile t - NSTAGE have been, and if that tile had not
+    // landed all CW warps would be waiting for it.  This takes a slice for every warp: with
+    // fewer, the spare warps run round the ring.  Without claims a warp has read its own
+    // slice of tile t - NSTAGE.
     constexpr bool CLAIM = FK == FK_SOA;
     for (unsigned it = 0;; ++it) {
-        unsigned g = it * TMA_CONSUMER_WARPS + (unsigned)warp;
+        unsigned t = it;
+        int sl = warp;
         if constexpr (CLAIM) {
-            g = claim_slice(slice_ctr, lane);
+            const unsigned g = claim_slice(slice_ctr, lane);
+            t = g / CW;
+            sl = (int)(g % CW);
         }
-        const unsigned t = g / SLICES;
-        const int sl = (int)(g % SLICES);
         const int64_t tile = blockIdx.x + (int64_t)t * gridDim.x;
         if (tile >= ntiles) break;
         const int s = (int)(t % TMA_NSTAGE);
