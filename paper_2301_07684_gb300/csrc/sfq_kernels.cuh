@@ -285,13 +285,10 @@ __device__ __forceinline__ T ln_spectrum(const T *__restrict__ k23, const T *__r
 // du/dt = q (E + u x B / gamma), q in units of |e|.
 //   u- = u + q E dt/2;  t = q B dt / (2 gamma(u-));  s = 2 t / (1 + t.t);
 //   u' = u- + u- x t;  u+ = u- + u' x s;  u_new = u+ + q E dt/2.
-// h / sqrt(g2) and 2 / d, both arguments at least 1.  The binary64 push is bound by the FP64 pipe
-// (86 % busy): one reciprocal root instead of a root and a division, and 2 / d from rcp_nr
-// (within 0.5 ulp, as the division) take 1.2e6 particles from 134 to 111 us.
+// h / sqrt(g2), g2 at least 1.  The binary64 push is bound by the FP64 pipe: one reciprocal root
+// instead of a root and a division.
 __device__ __forceinline__ float boris_h(float h, float g2) { return h / sqrtf(g2); }
-__device__ __forceinline__ float boris_f(float d) { return 2.0f / d; }
 __device__ __forceinline__ double boris_h(double h, double g2) { return h * rsqrt_nr(g2); }
-__device__ __forceinline__ double boris_f(double d) { return 2.0 * rcp_nr(d); }
 template <typename T>
 __device__ __forceinline__ void boris(T u[3], const T E[3], const T B[3], T q, T dt) {
     const T h = (T)0.5 * q * dt;
@@ -301,7 +298,7 @@ __device__ __forceinline__ void boris(T u[3], const T E[3], const T B[3], T q, T
     const T hg = boris_h(h, fma(um[0], um[0], fma(um[1], um[1], fma(um[2], um[2], (T)1))));
 #pragma unroll
     for (int k = 0; k < 3; ++k) t[k] = hg * B[k];
-    const T f = boris_f(fma(t[0], t[0], fma(t[1], t[1], fma(t[2], t[2], (T)1))));
+    const T f = (T)2 / fma(t[0], t[0], fma(t[1], t[1], fma(t[2], t[2], (T)1)));
 #pragma unroll
     for (int k = 0; k < 3; ++k) s[k] = f * t[k];
     const T c0 = um[1] * t[2] - um[2] * t[1], c1 = um[2] * t[0] - um[0] * t[2], c2 = um[0] * t[1] - um[1] * t[0];
