@@ -285,17 +285,13 @@ __device__ __forceinline__ T ln_spectrum(const T *__restrict__ k23, const T *__r
 // du/dt = q (E + u x B / gamma), q in units of |e|.
 //   u- = u + q E dt/2;  t = q B dt / (2 gamma(u-));  s = 2 t / (1 + t.t);
 //   u' = u- + u- x t;  u+ = u- + u' x s;  u_new = u+ + q E dt/2.
-// h / sqrt(g2), g2 at least 1.  The binary64 push is bound by the FP64 pipe: one reciprocal root
-// instead of a root and a division.
-__device__ __forceinline__ float boris_h(float h, float g2) { return h / sqrtf(g2); }
-__device__ __forceinline__ double boris_h(double h, double g2) { return h * rsqrt_nr(g2); }
 template <typename T>
 __device__ __forceinline__ void boris(T u[3], const T E[3], const T B[3], T q, T dt) {
     const T h = (T)0.5 * q * dt;
     T um[3], t[3], s[3], up[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) um[k] = fma(h, E[k], u[k]);
-    const T hg = boris_h(h, fma(um[0], um[0], fma(um[1], um[1], fma(um[2], um[2], (T)1))));
+    const T hg = h / sqrt(fma(um[0], um[0], fma(um[1], um[1], fma(um[2], um[2], (T)1))));
 #pragma unroll
     for (int k = 0; k < 3; ++k) t[k] = hg * B[k];
     const T f = (T)2 / fma(t[0], t[0], fma(t[1], t[1], fma(t[2], t[2], (T)1)));

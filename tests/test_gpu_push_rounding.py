@@ -1,4 +1,6 @@
-"""The binary64 push's arithmetic: its factors where their argument overflows."""
+"""The binary64 push's arithmetic: its factors' bits, and where their argument overflows."""
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -34,3 +36,19 @@ def test_rotation_by_a_field_whose_square_overflows():
     assert np.abs(x / want - 1).max() < 20 * 2.0 ** -53, x
     assert np.abs(y / px).max() < 20 * 2.0 ** -53, y
     assert np.array_equal(z, np.full(6, 0.5))
+
+
+def test_factors_are_rounded_as_the_formula_says():
+    """With u = (1, 0, pz) and B along z, u_y = -s = -2 t / (1 + t^2), t = h B / gamma: every
+    operation of it is correctly rounded (root, divisions, products, 1 + t^2 with one
+    rounding), so the result has the bits of the same operations on the host."""
+    g = np.random.default_rng(3)
+    n = 20000
+    pz, bz = 10.0 ** g.uniform(-2, 5, n), 10.0 ** g.uniform(-2, 6, n)
+    pz[: n // 2] = 0.0                                     # gamma^2 = 2
+    _, y, _ = _push(np.ones(n), pz, bz, 2.0)
+    one_plus_square = np.array([float(1 + Fraction(v) ** 2) for v in pz.tolist()])
+    g2 = np.array([float(1 + Fraction(v)) for v in one_plus_square.tolist()])
+    t = (1.0 / np.sqrt(g2)) * bz
+    d = np.array([float(1 + Fraction(v) ** 2) for v in t.tolist()])
+    assert np.array_equal(y, -((2.0 / d) * t))
