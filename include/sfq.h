@@ -386,9 +386,11 @@ sfq_status sfq_autotune_step(sfq_ctx *ctx, const sfq_particles *p, const sfq_fie
 /* Sort the first n product records in place by (parent id, step, member, parent tag)
  * (a stable LSD radix sort).  `scratch` is caller-owned device memory of at least
  * sfq_sort_scratch_bytes(n) bytes, 256-byte aligned; nothing in it needs to start at zero.
- * Synchronises `stream` at most once (large sorts read back which key bits differ between
- * records; only those are sorted).  Returns SFQ_ERR_ARG if scratch is NULL, misaligned or
- * too small, or if n exceeds the capacity of `out` or 2^32 - 1. */
+ * For n > 1 it synchronises `stream` once, before records are moved (large sorts read back
+ * which key bits differ between records; only those are sorted): on return the work queued
+ * on `stream` before the call has finished, and the sort itself may still be running.
+ * Returns SFQ_ERR_ARG if scratch is NULL, misaligned or too small, or if n exceeds the
+ * capacity of `out` or 2^32 - 1. */
 size_t sfq_sort_scratch_bytes(int64_t n);
 sfq_status sfq_sort_products(sfq_ctx *ctx, const sfq_products *out, int64_t n, void *scratch, size_t scratch_bytes,
                              void *stream);
@@ -406,7 +408,7 @@ sfq_status sfq_sort_products(sfq_ctx *ctx, const sfq_products *out, int64_t n, v
  *   The first call with each context looks up the array's address on the context's device
  *   (cudaGetSymbolAddress) and keeps it in the context; make that first call before any
  *   stream capture begins.
- *   Synchronises `stream` at most once, as sfq_sort_products does. */
+ *   Synchronises `stream` once, as sfq_sort_products does. */
 #define SFQ_SORT_NOALLOC_MAX_N (1 << 20)
 #define SFQ_SORT_NOALLOC_SCRATCH_BYTES (44u << 20)
 sfq_status sfq_sort_products_noalloc(sfq_ctx *ctx, const sfq_products *out, int64_t n, void *stream);

@@ -579,7 +579,14 @@ cudaError_t sort_products(const sfq_products &out, int64_t n, size_t elem, void 
     cudaError_t e = cudaStreamIsCapturing(s, &cap);
     if (e != cudaSuccess) return e;
     if (cap != cudaStreamCaptureStatusNone) return cudaErrorStreamCaptureUnsupported;
-    if (n <= SMALL_N) return elem == 4 ? small_sort<float>(out, (int)n, s) : small_sort<double>(out, (int)n, s);
+    if (n <= SMALL_N) {
+        // every sort waits for the stream's earlier work: the larger ones by their read-back, this
+        // one only because callers rely on it (a step loop has read the record count by now and
+        // finds the stream idle)
+        e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return e;
+        return elem == 4 ? small_sort<float>(out, (int)n, s) : small_sort<double>(out, (int)n, s);
+    }
     const Plan P = plan(n);
     char *sc = static_cast<char *>(scratch);
     Bits *bits = reinterpret_cast<Bits *>(sc + P.o_bits);
