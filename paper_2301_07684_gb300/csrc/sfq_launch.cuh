@@ -92,16 +92,6 @@ static cudaError_t launch_uniforms_t(int64_t n, const uint64_t *id, uint32_t ste
 
 // Dynamic shared-memory limits of the TMA-staged kernels, set once per process (and before
 // any stream capture, where the launch itself is recorded).
-// The TMA-staged shapes compiled with the truncated samplers (TRUNC) are limited to 16
-// consumer warps; the warp-streaming ones to 2 particles per lane.
-constexpr int TRUNC_CW = 16, TRUNC_PPT = 2;
-// Consumer warps per block of the default binary32 shapes.  With the producer they are 20 or 16 warps, 5
-// or 4 per scheduler, which leaves 96 or 128 registers a thread (16 consumer warps: 17, five
-// on one scheduler).  Fields in memory wait on HBM and on event batches, where more warps
-// help: 8 steps of 2^24 particles 1539 us with 19, 1552 with 15, 1574 with 23 (80 registers).
-// The plane wave is bound by issue: 40 steps of 4.2e6 particles 2058 us with 15, 2085 with 19,
-// 2191 with 23.
-constexpr int TMA_CW_SOA = 19, TMA_CW_PW = 15;
 
 template <typename T, bool TRUNC>
 static cudaError_t prepare_step_t() {
@@ -229,7 +219,8 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
     //    particles gains from more (507 / 493 us at 4*10^6).
     const bool f64 = sizeof(T) == 8;
     const int dflt = f64 ? (pw && p.n >= (1ll << 21) ? TMA_CW_PW : 8) : (pw ? TMA_CW_PW : TMA_CW_SOA);
-    const int cw = TRUNC ? TRUNC_CW : ((L.ppt == 8 || L.ppt == 16 || L.ppt == 20) ? L.ppt : dflt);
+    const bool given = L.ppt == 8 || L.ppt == 16 || L.ppt == 20 || (pw ? L.ppt == TMA_CW_PW : !f64 && L.ppt == TMA_CW_SOA);
+    const int cw = TRUNC ? TRUNC_CW : (given ? L.ppt : dflt);
     const int tile = cw * (f64 ? 32 : 64);
     const int64_t tma_from = (int64_t)(TRUNC ? tile : (f64 ? 128 : (pw ? 1024 : 10 * 1024))) * ctx->num_sms;
     // the beyond-LCFA model runs on the warp-streaming kernel (its state is read directly)

@@ -219,8 +219,17 @@ sfq_status sfq_autotune_step(sfq_ctx *ctx, const sfq_particles *p, const sfq_fie
         return st;
     }
     struct Shape { int variant, ppt; };
-    const Shape shapes[7] = {{1, 1}, {1, 2}, {1, 4}, {2, 8}, {2, 16}, {2, 20}, {2, 0}};
-    const int nshapes = blcfa ? 3 : 7;           // the beyond-LCFA model runs on the warp-streaming kernel
+    // every shape that the step compiles for this precision and field source, named by its warps:
+    // what is timed on the sample is what the population then runs.  The beyond-LCFA model
+    // runs on the warp-streaming kernel; the truncated samplers have one shape of each kernel.
+    Shape shapes[7];
+    int nshapes = 0;
+    const bool trunc = ctx->inv_tr > 0;
+    for (int k : {1, 2, 4})
+        if (!trunc || k == sfq::TRUNC_PPT) shapes[nshapes++] = {1, k};
+    const int own = f->kind == SFQ_FIELDS_PLANE_WAVE ? sfq::TMA_CW_PW : (fp64 ? 0 : sfq::TMA_CW_SOA);
+    for (int k : {8, 16, 20, own})
+        if (!blcfa && k && (!trunc || k == sfq::TRUNC_CW)) shapes[nshapes++] = {2, k};
     const int saved[3] = {ctx->step_variant, ctx->step_ppt, ctx->step_grid};
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     e = cudaEventCreate(&ev0);
