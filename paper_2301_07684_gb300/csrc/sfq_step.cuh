@@ -119,24 +119,26 @@ __device__ __forceinline__ void load_fields(const StepArgs<T> &a, int64_t i, T E
     }
 }
 
-// chi rho = sqrt((gamma E + p x B)^2 - (p.E)^2): Eq. chi_exact multiplied through by gamma.
-template <typename T>
-__device__ __forceinline__ T chi_of(T g, T px, T py, T pz, const T E[3], const T B[3], T inv_rho) {
-    const T fx = fma(g, E[0], py * B[2] - pz * B[1]);
-    const T fy = fma(g, E[1], pz * B[0] - px * B[2]);
-    const T fz = fma(g, E[2], px * B[1] - py * B[0]);
-    const T pe = fma(px, E[0], fma(py, E[1], pz * E[2]));
-    const T q = fma(fx, fx, fma(fy, fy, fz * fz)) - pe * pe;
-    return sqrt_nr(q) * inv_rho;
-}
-
-// chi in the linearly polarised plane wave E = (0, f, 0), B = (0, 0, f): Eq. chi_exact with
-// the vanishing components dropped (gamma E + p x B = (py f, gamma f - px f, 0), p.E = py f).
-// Every operation is rounded explicitly, so all kernels form the same bits.
+// Every operation of chi_of and chi_pw is rounded explicitly, so all kernels form the same bits
+// (step_pair writes the same operations on packed registers).
 __device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
 __device__ __forceinline__ double mul_rn(double x, double y) { return __dmul_rn(x, y); }
 __device__ __forceinline__ float sub_rn(float x, float y) { return __fsub_rn(x, y); }
 __device__ __forceinline__ double sub_rn(double x, double y) { return __dsub_rn(x, y); }
+
+// chi rho = sqrt((gamma E + p x B)^2 - (p.E)^2): Eq. chi_exact multiplied through by gamma.
+template <typename T>
+__device__ __forceinline__ T chi_of(T g, T px, T py, T pz, const T E[3], const T B[3], T inv_rho) {
+    const T fx = fma(g, E[0], fma(py, B[2], mul_rn(-pz, B[1])));
+    const T fy = fma(g, E[1], fma(pz, B[0], mul_rn(-px, B[2])));
+    const T fz = fma(g, E[2], fma(px, B[1], mul_rn(-py, B[0])));
+    const T pe = fma(px, E[0], fma(py, E[1], mul_rn(pz, E[2])));
+    const T q = fma(-pe, pe, fma(fx, fx, fma(fy, fy, mul_rn(fz, fz))));
+    return mul_rn(sqrt_nr(q), inv_rho);
+}
+
+// chi in the linearly polarised plane wave E = (0, f, 0), B = (0, 0, f): Eq. chi_exact with
+// the vanishing components dropped (gamma E + p x B = (py f, gamma f - px f, 0), p.E = py f).
 template <typename T>
 __device__ __forceinline__ T chi_pw(T g, T px, T py, T f, T inv_rho) {
     const T fx = mul_rn(py, f);
