@@ -97,9 +97,6 @@ constexpr int STEP_BS = 256;
 #ifndef SFQ_STEP_MINB
 #define SFQ_STEP_MINB 4   // resident blocks per SM the register allocation aims for (measured best)
 #endif
-#ifndef SFQ_LEPTON_MINB
-#define SFQ_LEPTON_MINB 4 // the same for the beyond-LCFA lepton and full-cascade instances
-#endif
 
 enum { FK_SOA = 0, FK_PW = 1 };
 
@@ -763,11 +760,10 @@ __device__ __forceinline__ void step_pair(const StepArgs<float> &a, const float 
 // warp-private ring in shared memory; a full batch of 32 events is sampled by the
 // whole warp.  No block-wide barrier inside the loop.
 // CASC: the full-cascade instance (every product is also spawned, with its own id).
-// MINB: resident blocks per SM the register allocation aims for (the beyond-LCFA lepton and
-// full-cascade instances take SFQ_LEPTON_MINB: their event paths hold more state).
-template <typename T, int FK, int PPT, bool TRUNC = false, bool CASC = false, bool SURR = false,
-          int MINB = SFQ_STEP_MINB>
-__global__ void __launch_bounds__(STEP_BS, MINB) mc_step_kernel(const StepArgs<T> a) {
+// One instance serves LCFA and beyond-LCFA leptons (a test of the model at run time); the
+// latter's state makes it spill at the registers that SFQ_STEP_MINB blocks leave.
+template <typename T, int FK, int PPT, bool TRUNC = false, bool CASC = false, bool SURR = false>
+__global__ void __launch_bounds__(STEP_BS, SFQ_STEP_MINB) mc_step_kernel(const StepArgs<T> a) {
     using Q = L<T>;
     constexpr int WARPS = STEP_BS / 32;
     constexpr int QS = (32 * (PPT + 1) <= 64) ? 64 : ((32 * (PPT + 1) <= 128) ? 128 : 256);
