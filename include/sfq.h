@@ -530,10 +530,9 @@ sfq_status sfq_set_event_queue(sfq_ctx *ctx, const sfq_event_queue *queue);
  *            memory, one persistent block per SM).
  *   ppt:     shape of the chosen kernel: particles per lane per chunk of the
  *            warp-streaming kernel (1, 2 or 4), or consumer warps per block of the
- *            TMA-staged kernel: 8, 16 or 20, 15 (plane wave; the default shape with
- *            fields in memory) or 19 (fields in memory; the default shape with the plane
- *            wave; binary32 contexts only); 0 = default, chosen by precision and field
- *            source, for a binary64 plane wave also by the population's size.
+ *            TMA-staged kernel: 8, 16, 20 or 15 (plane wave; the default shape with
+ *            fields in memory); 0 = default, chosen by precision and field source, for a
+ *            binary64 plane wave also by the population's size.
  *   grid_blocks: grid size (0 = one wave of resident blocks on every SM).
  * Returns SFQ_ERR_ARG for other values.  Results do not depend on the shape. */
 sfq_status sfq_set_step_shape(sfq_ctx *ctx, int32_t variant, int32_t ppt, int32_t grid_blocks);

@@ -524,12 +524,10 @@ sfq_status sfq_sampler_coefficients(const sfq_ctx *ctx, int32_t *n, int32_t *k) 
 sfq_status sfq_set_step_shape(sfq_ctx *ctx, int32_t variant, int32_t ppt, int32_t grid_blocks) {
     if (!ctx) return SFQ_ERR_ARG;
     if (variant < 0 || variant > 2) return fail(ctx, SFQ_ERR_ARG, "variant must be 0, 1 or 2");
-    const bool ok = variant == 2 ? (ppt == 0 || ppt == 8 || ppt == 16 || ppt == 20 || ppt == sfq::TMA_CW_PW ||
-                                    (ppt == sfq::TMA_CW_SOA && !is_fp64(ctx)))
+    const bool ok = variant == 2 ? (ppt == 0 || ppt == 8 || ppt == 16 || ppt == 20 || ppt == sfq::TMA_CW_PW)
                                  : (ppt == 0 || ppt == 1 || ppt == 2 || ppt == 4);
     if (!ok)
-        return fail(ctx, SFQ_ERR_ARG,
-                    "shape: 1, 2 or 4 particles per lane (variant 1), 8/15/16/20 or (binary32) 19 warps (variant 2)");
+        return fail(ctx, SFQ_ERR_ARG, "shape: 1, 2 or 4 particles per lane (variant 1), 8/15/16/20 warps (variant 2)");
     if (grid_blocks < 0) return fail(ctx, SFQ_ERR_ARG, "grid_blocks < 0");
     ctx->step_variant = variant;
     ctx->step_ppt = ppt;

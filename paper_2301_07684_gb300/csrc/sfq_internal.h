@@ -39,13 +39,12 @@ struct sfq_ctx {
 
 namespace sfq {
 
-// Consumer warps per block of the default binary32 shapes.  With the producer they are 20 or
-// 16 warps, 5 or 4 per scheduler, which leaves 96 or 128 registers a thread (16 consumer
-// warps: 17, five on one scheduler).  Fields in memory wait on HBM and on event batches, where more warps
-// help: 8 steps of 2^24 particles 1539 us with 19, 1552 with 15, 1574 with 23 (80 registers).
-// The plane wave is bound by issue: 40 steps of 4.2e6 particles 2058 us with 15, 2085 with 19,
-// 2191 with 23.
-constexpr int TMA_CW_SOA = 19, TMA_CW_PW = 15;
+// Consumer warps per block of the default binary32 shapes: 8 steps of 2^24 particles with
+// fields in memory take 1533 us with 16, 1542 with 19, 1812 with 20 (two stages fit) and 2110
+// with 8; 40 steps of 4.2e6 particles in the plane wave 2076 us with 15, 2088 with 16, 2168
+// with 20 and 2749 with 8 (15 and the producer are four warps per scheduler, which leaves
+// 128 registers a thread).
+constexpr int TMA_CW_SOA = 16, TMA_CW_PW = 15;
 // The TMA-staged shapes compiled with the truncated samplers (TRUNC) are limited to 16
 // consumer warps; the warp-streaming ones to 2 particles per lane.
 constexpr int TRUNC_CW = 16, TRUNC_PPT = 2;

@@ -92,7 +92,6 @@ static cudaError_t launch_uniforms_t(int64_t n, const uint64_t *id, uint32_t ste
 
 // Dynamic shared-memory limits of the TMA-staged kernels, set once per process (and before
 // any stream capture, where the launch itself is recorded).
-
 template <typename T, bool TRUNC>
 static cudaError_t prepare_step_t() {
     static bool done = false;
@@ -111,12 +110,6 @@ static cudaError_t prepare_step_t() {
         SFQ_PREP(8)
         SFQ_PREP(16)
         SFQ_PREP(20)
-        if constexpr (sizeof(T) == 4) {
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>());
-        }
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(mc_step_tma_kernel<T, FK_PW, TMA_CW_PW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)tma_smem_bytes<T, FK_PW, TMA_CW_PW>());
@@ -209,17 +202,18 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
     // TMA-staged kernel: one persistent block per SM; `ppt` selects the consumer warps per block.
     // Chosen automatically (us per step in a graph, warp-streaming against TMA-staged):
     //  - binary32, fields in memory: from ten tiles per SM, where the pipeline has filled (150,000
-    //    particles 10.9 / 12.5, 300,000 13.6 / 16.3, 10^6 19.4 / 20.8, 2*10^6 33.2 / 29.3);
+    //    particles 13.0 / 14.0, 300,000 16.0 / 16.0, 10^6 22.0 / 23.8, 1.5*10^6 27.9 / 27.3,
+    //    2*10^6 36.2 / 32.4);
     //  - binary32, plane wave: from a tile per SM (11.1 / 11.9 at 150,000, 13.8 / 13.6 at 300,000,
     //    31.6 / 30.6 at 2*10^6);
     //  - binary64: from 128 particles per SM (28 / 27 at 20,000, 80 / 44 at 160,000, 556 / 532 at
     //    4*10^6), with 8 consumer warps: the FP64 pipe takes two lanes per clock and SM whatever
     //    a warp's active lanes, 8 warps keep it busy and leave 8 partial event batches at the
-    //    end instead of 16 (62) or 19 (67 us at 160,000).  Only a plane wave of millions of
+    //    end instead of 16 (62 us at 160,000).  Only a plane wave of millions of
     //    particles gains from more (507 / 493 us at 4*10^6).
     const bool f64 = sizeof(T) == 8;
     const int dflt = f64 ? (pw && p.n >= (1ll << 21) ? TMA_CW_PW : 8) : (pw ? TMA_CW_PW : TMA_CW_SOA);
-    const bool given = L.ppt == 8 || L.ppt == 16 || L.ppt == 20 || (pw ? L.ppt == TMA_CW_PW : !f64 && L.ppt == TMA_CW_SOA);
+    const bool given = L.ppt == 8 || L.ppt == 16 || L.ppt == 20 || (pw && L.ppt == TMA_CW_PW);
     const int cw = TRUNC ? TRUNC_CW : (given ? L.ppt : dflt);
     const int tile = cw * (f64 ? 32 : 64);
     const int64_t tma_from = (int64_t)(TRUNC ? tile : (f64 ? 128 : (pw ? 1024 : 10 * 1024))) * ctx->num_sms;
@@ -242,18 +236,13 @@ static cudaError_t launch_step_t(const StepLaunch &L) {
         } else {
             switch (cw) {
                 SFQ_TMA_CASE(8)
-                SFQ_TMA_CASE(16)
                 SFQ_TMA_CASE(20)
                 case TMA_CW_PW:
                     kern = mc_step_tma_kernel<T, FK_PW, TMA_CW_PW>;
                     smem = tma_smem_bytes<T, FK_PW, TMA_CW_PW>();
                     break;
                 default:
-                    if constexpr (sizeof(T) == 4) {
-                        kern = mc_step_tma_kernel<T, FK_SOA, TMA_CW_SOA>;
-                        smem = tma_smem_bytes<T, FK_SOA, TMA_CW_SOA>();
-                    }
-                    break;
+                SFQ_TMA_CASE(16)
             }
         }
 #undef SFQ_TMA_CASE

@@ -227,7 +227,7 @@ sfq_status sfq_autotune_step(sfq_ctx *ctx, const sfq_particles *p, const sfq_fie
     const bool trunc = ctx->inv_tr > 0;
     for (int k : {1, 2, 4})
         if (!trunc || k == sfq::TRUNC_PPT) shapes[nshapes++] = {1, k};
-    const int own = f->kind == SFQ_FIELDS_PLANE_WAVE ? sfq::TMA_CW_PW : (fp64 ? 0 : sfq::TMA_CW_SOA);
+    const int own = f->kind == SFQ_FIELDS_PLANE_WAVE ? sfq::TMA_CW_PW : 0;
     for (int k : {8, 16, 20, own})
         if (!blcfa && k && (!trunc || k == sfq::TRUNC_CW)) shapes[nshapes++] = {2, k};
     const int saved[3] = {ctx->step_variant, ctx->step_ppt, ctx->step_grid};
