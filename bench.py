@@ -1114,7 +1114,7 @@ def main():
     ap.add_argument("--min-timed-ms", type=float, default=1500.0,
                     help="add regions until this much timed work (so the clock sampler sees the region)")
     ap.add_argument("--oracle-steps", type=int, default=50)
-    # DRAM bytes (read + write) per update of mc_step_tma_kernel<float, SoA, 19 warps>, from the
+    # DRAM bytes (read + write) per update of mc_step_tma_kernel<float, SoA, 16 warps>, from the
     # ncu capture summarised in profiles/mc_step_tma_fp32_soa_4M.md (4,194,304 particles;
     # the per-particle streams scale in proportion to n).  Re-measure whenever that kernel
     # changes, and pass --traffic-per-update 0 to report null meanwhile.
@@ -1122,7 +1122,7 @@ def main():
                     help="FP64-pipe instructions per update of the binary64 step kernel (ncu capture)")
     ap.add_argument("--fp64-pipe-busy", type=float, default=0.884,
                     help="sm__pipe_fp64_cycles_active of the binary64 step kernel (ncu capture)")
-    ap.add_argument("--traffic-per-update", type=float, default=51.31,
+    ap.add_argument("--traffic-per-update", type=float, default=51.23,
                     help="DRAM bytes per update of the step kernel from an ncu capture (for roofline.traffic)")
     args = ap.parse_args()
     args.warmup = max(3, args.warmup)

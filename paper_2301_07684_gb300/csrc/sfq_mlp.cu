@@ -433,7 +433,9 @@ __device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
     return __uint_as_float(r);
 }
 // Row m of a 128 x 64 (or 64 x 64) K-major operand: 8 chunks of 8 bf16 (16 bytes).
-__device__ __forceinline__ uint32_t row_chunk_offset(int m, int j) { return (uint32_t)((((m >> 3) * 8) + j) * 128 + (m & 7) * 16); }
+__device__ __forceinline__ uint32_t row_chunk_offset(int m, int j) {
+    return (uint32_t)((((m >> 3) * 8) + j) * 128 + (m & 7) * 16);
+}
 // The finishing of queued photon emissions (APPLY): the emitter's state before the event,
 // its population, and the product records (sfq_set_surrogate).
 struct ApplyOut {
@@ -487,7 +489,8 @@ constexpr uint32_t INFER_SMEM = SM_BYTES + 128;      // + alignment slack
 #ifndef SFQ_INFER_MINB
 #define SFQ_INFER_MINB 4
 #endif
-constexpr int INFER_MINB = SFQ_INFER_MINB;            // resident blocks per SM (registers, 53 KB of shared memory, 128 of 512 TMEM columns each)
+// resident blocks per SM (registers, 53 KB of shared memory, 128 of 512 TMEM columns each)
+constexpr int INFER_MINB = SFQ_INFER_MINB;
 
 // SiLU of two units in packed registers: silu_h for each, one multiply-add for both.
 __device__ __forceinline__ f32x2 silu_h2(f32x2 h) {

@@ -204,11 +204,10 @@ struct ScatterSmem {
     K key[TILE];
 };
 template <typename K>
-__global__ void __launch_bounds__(SB, sizeof(K) == 4 ? 1024 / SB : 512 / SB) sort_scatter_kernel(int64_t n, const K *__restrict__ key_in,
-                                                          const uint32_t *__restrict__ idx_in, K *__restrict__ key_out,
-                                                          uint32_t *__restrict__ idx_out, int shift,
-                                                          const uint32_t *__restrict__ counts, int ntiles,
-                                                          const uint32_t *__restrict__ total) {
+__global__ void __launch_bounds__(SB, sizeof(K) == 4 ? 1024 / SB : 512 / SB)
+    sort_scatter_kernel(int64_t n, const K *__restrict__ key_in, const uint32_t *__restrict__ idx_in,
+                        K *__restrict__ key_out, uint32_t *__restrict__ idx_out, int shift,
+                        const uint32_t *__restrict__ counts, int ntiles, const uint32_t *__restrict__ total) {
     extern __shared__ __align__(16) unsigned char smraw[];
     ScatterSmem<K> &S = *reinterpret_cast<ScatterSmem<K> *>(smraw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -337,8 +336,8 @@ __global__ void gather_kernel(int64_t n, const uint32_t *__restrict__ perm, cons
 // ---------------------------------------------------------------------------
 // Up to SMALL_N records in one block: a step loop's few thousand photons, where the launches
 // and the read-back of the general path are what a caller waits for.  A call with 1000 / 8000 /
-// 16384 records takes 44 / 65 / 96 us from Python, 79 / 106 / 106 us through the general path
-// (226 / 254 / 248 us before either), so the line is where one SM's latency meets it.
+// 16384 records takes 37 / 59 / 91 us from Python, 74 / 77 / 100 us through the general path,
+// so the line is where one SM's latency meets it.
 constexpr int SMALL_N = 16384, MB = 1024, MW = MB / 32, MR = SMALL_N / MB;
 static_assert(SMALL_N <= 1 << 14 && SMALL_N / MW <= 1 << 9, "index, digit and rank share a word");
 struct SmallSmem {

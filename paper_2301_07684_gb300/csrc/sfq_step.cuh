@@ -569,9 +569,9 @@ __device__ __forceinline__ void process_events(const StepArgs<T> &a, int64_t ei,
 }
 
 // Comparisons of the update: binary64 ones on the bit patterns, by the integer pipe (a binary64
-// comparison takes the FP64 pipe, which bounds that path, as long as a multiply-add; with
-// the push's divisions, 4 pushes and steps of 1.2e6 particles 1568 -> 1408 us).  x >= 0 of a value that is never
-// -0, x > 0, x > 0.1; false for NaN.
+// comparison takes the FP64 pipe, which bounds that path, as long as a multiply-add: 4 pushes
+// and steps of 1.2e6 particles with their sort take 1482 us, 1533 with binary64 ones).
+// x >= 0 of a value that is never -0, x > 0, x > 0.1; false for NaN.
 __device__ __forceinline__ bool not_negative(float x) { return x >= 0.0f; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.0f; }
 __device__ __forceinline__ bool above_tenth(float x) { return x > 0.1f; }

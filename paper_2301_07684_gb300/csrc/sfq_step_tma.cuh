@@ -11,11 +11,13 @@
 // samples them 32 at a time.
 // What bounds it (binary32): with fields in memory 53 B per particle from and to HBM, about
 // 59 with the 32-byte sectors of the momenta that events rewrite; 2^24 particles take 175 us
-// (190 with two scalar particles per lane), 83 % of the copy bandwidth on those bytes.  The plane wave, and populations too small to
-// fill the stages many times, are bound by issue: two leptons of a lane are stepped in
-// packed registers without branches (step_pair), 6.5 warp-instructions per particle
-// with its events (8.2 before, when 4.2e6 particles took 57 us under the profiler with fields
-// in memory and 57 with the wave; now 45 and 47).  Stages are handed over with mbarriers
+// (190 with two scalar particles per lane), 83 % of the copy bandwidth on those bytes.  The
+// plane wave moves 35 B and takes as long: it waits.  Of 2^22 particles (under the profiler)
+// it steps one in 6.8 warp-instructions with its events and uses 50 % of the issue slots; per
+// issue its warps stall 1.9 cycles on loads of events and of the wave's table and 1.8 on
+// fixed latencies (55 us; fields in memory: 7.0, 54 %, 1.3 and 1.8, 52 us; 8.2 and 59 us
+// scalar).  Two leptons of a lane are stepped in packed registers without branches
+// (step_pair).  Stages are handed over with mbarriers
 // (full: producer -> consumers, completed by the copies' transaction bytes;
 // empty: consumers -> producer).  Every wait is bounded: on a timeout the kernel
 // raises the timeout word of the counters and leaves its loops after its copies

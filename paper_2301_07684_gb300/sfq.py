@@ -186,7 +186,7 @@ EXPORTED = ["sfq_init", "sfq_finalize", "sfq_last_error", "sfq_constants", "sfq_
 # A step call marshals about forty pointers and numbers; for a small population that, not the
 # kernel, is what the call takes.  So addresses go to ctypes as plain integers, descriptors are
 # built in one call each, and the stream's handle is read without a torch.cuda.Stream object
-# (16 steps of 10,007 particles and their sort: 340 us before, 259 us so).
+# (16 steps of 10,007 particles and their sort: 340 us before, 264 us so).
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
